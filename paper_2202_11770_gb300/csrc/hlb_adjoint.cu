@@ -115,39 +115,13 @@ __device__ __forceinline__ R block_sum_r(R v, R* sh) {
 // fluid and i is odd or the link is not fluid and i is even, and off[i] - n
 // otherwise (mu_offset), so one decode of the index serves both gathers.
 template <bool CT, bool WIDE>
-__device__ __forceinline__ void reverse_offsets(const int32_t* __restrict__ src, const uint32_t* __restrict__ ctab,
-                                                const int32_t* __restrict__ tbase, uint32_t sn, uint32_t n,
-                                                uint32_t x, uint32_t tile, uint32_t* off, uint32_t* fluid) {
+__device__ __forceinline__ void reverse_offsets(const IndexTables& ix, uint32_t sn, uint32_t n, uint32_t x, uint32_t tile,
+                                                uint32_t* off, uint32_t* fluid) {
   uint32_t fl = 0;
-  if (CT) {
-    uint32_t w[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) w[q] = __ldg(WIDE ? ctab + ((uint64_t)q * sn + x) : ctab + (uint32_t)q * sn + x);
-    const int4* tb = reinterpret_cast<const int4*>(tbase + (uint64_t)tile * CT_BASES);
-    int b[20];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const int4 v = __ldg(tb + q);
-      b[4 * q] = v.x;
-      b[4 * q + 1] = v.y;
-      b[4 * q + 2] = v.z;
-      b[4 * q + 3] = v.w;
-    }
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const uint32_t o = (i & 1) ? (w[(i - 1) >> 1] & 0xffffu) : (w[(i - 1) >> 1] >> 16);
-      const bool f = o < CT_IOLET;
-      off[i] = f ? slot<WIDE>(i, n, (uint32_t)b[i - 1] + o) : slot<WIDE>(opp(i), n, x);
-      fl |= f ? 1u << i : 0u;
-    }
-  } else {
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const int32_t s = __ldg(idx_at<WIDE>(src, i, sn, x));
-      off[i] = s >= 0 ? slot<WIDE>(i, n, (uint32_t)s) : slot<WIDE>(opp(i), n, x);
-      fl |= s >= 0 ? 1u << i : 0u;
-    }
-  }
+  for_links<CT, WIDE, LD_NC, false>(ix, sn, x, tile, [&](int i, bool f, uint32_t s) {
+    off[i] = f ? slot<WIDE>(i, n, s) : slot<WIDE>(opp(i), n, x);
+    fl |= f ? 1u << i : 0u;
+  });
   *fluid = fl;
 }
 __device__ __forceinline__ uint32_t mu_offset(uint32_t off, uint32_t fluid, int i, uint32_t n) {
@@ -171,10 +145,7 @@ __device__ __forceinline__ uint32_t mu_offset(uint32_t off, uint32_t fluid, int 
 // and the index rows staged in shared memory with bulk copies.
 template <typename S, bool GPREV, bool WIDE, bool CT>
 __device__ __forceinline__ typename Real<S>::type adjoint_site(const S* __restrict__ prev, const S* __restrict__ mu_next,
-                                                               S* __restrict__ mu_out, const int32_t* __restrict__ src,
-                                                               const uint32_t* __restrict__ ctab,
-                                                               const int32_t* __restrict__ tbase,
-                                                               const uint32_t* __restrict__ imask,
+                                                               S* __restrict__ mu_out, const IndexTables& ix,
                                                                const AdjParams& ap, const ProbeMap& pm, int store,
                                                                int64_t x, uint32_t tile,
                                                                typename Real<S>::type (*neq)[BLOCK]) {
@@ -182,9 +153,9 @@ __device__ __forceinline__ typename Real<S>::type adjoint_site(const S* __restri
   const uint32_t n = (uint32_t)ap.prev.n, sn = (uint32_t)ap.prev.sn, xi = (uint32_t)x;
   const R omega = omega_of<R>(ap.prev);
   if (x >= ap.prev.n) return R(0);
-  if ((__ldg(imask + (xi >> 5)) >> (xi & 31)) & 1u) return R(0);  // iolet sites: adjoint_iolet_site
+  if ((__ldg(ix.imask + (xi >> 5)) >> (xi & 31)) & 1u) return R(0);  // iolet sites: adjoint_iolet_site
   uint32_t off[Q], fluid;
-  reverse_offsets<CT, WIDE>(src, ctab, tbase, sn, n, xi, tile, off, &fluid);
+  reverse_offsets<CT, WIDE>(ix, sn, n, xi, tile, off, &fluid);
   pdl_wait();  // the states below were written by the kernels before this one
   pdl_trigger();
   R drho, rho, ux, uy, uz, usq15;
@@ -456,9 +427,7 @@ __device__ __forceinline__ typename Real<S>::type adjoint_iolet_site(const S* __
 template <typename S, bool GPREV, bool WIDE, bool CT>
 __global__ void __launch_bounds__(BLOCK, sizeof(typename Real<S>::type) == 8 ? 2 : 4)
     k_adjoint(const S* __restrict__ prev, const S* __restrict__ cur, const S* __restrict__ mu_next,
-              S* __restrict__ mu_out, const int32_t* __restrict__ src, const uint32_t* __restrict__ ctab,
-              const int32_t* __restrict__ tbase, const uint32_t* __restrict__ imask,
-              const LinkRec* __restrict__ links, const double* __restrict__ amp, const AdjParams ap,
+              S* __restrict__ mu_out, const IndexTables ix, const LinkRec* __restrict__ links, const double* __restrict__ amp, const AdjParams ap,
               const ProbeMap pm, const int32_t* __restrict__ sites, int64_t nsites, unsigned n_iolet_blocks,
               const BlockDiv stride, double* __restrict__ part, double* __restrict__ dlink, int store) {
   using R = typename Real<S>::type;
@@ -467,11 +436,11 @@ __global__ void __launch_bounds__(BLOCK, sizeof(typename Real<S>::type) == 8 ? 2
   const unsigned b = blockIdx.x, j = block_div(b, stride);
   R d;
   if (b == j * stride.d && j < n_iolet_blocks) {
-    d = adjoint_iolet_site<S, GPREV>(prev, cur, mu_next, mu_out, src, links, amp, ap, pm, sites, nsites, dlink,
+    d = adjoint_iolet_site<S, GPREV>(prev, cur, mu_next, mu_out, ix.src, links, amp, ap, pm, sites, nsites, dlink,
                                      store, ((int64_t)j * BLOCK + threadIdx.x) >> 5);
   } else {
     const unsigned k = b - min(n_iolet_blocks, j + 1);  // bulk block: blocks before b that are not iolet blocks
-    d = adjoint_site<S, GPREV, WIDE, CT>(prev, mu_next, mu_out, src, ctab, tbase, imask, ap, pm, store,
+    d = adjoint_site<S, GPREV, WIDE, CT>(prev, mu_next, mu_out, ix, ap, pm, store,
                                          (int64_t)k * BLOCK + threadIdx.x, k, neq);
   }
   // block sum of the dJ/dtau terms in the kernel's arithmetic type (FP64 on
@@ -552,8 +521,8 @@ cudaError_t launch_adjoint(const hlb_solver* h, const void* prev, bool gprev, co
   auto kernel = gprev ? pick(std::true_type{}) : pick(std::false_type{});
   // programmatic dependent launch: the index decode overlaps the previous
   // kernel's tail (the reverse steps and the segment recomputes alternate)
-  return launch_pdl(kernel, grid, BLOCK, st, (const S*)prev, (const S*)cur, (const S*)mu_next, (S*)mu_out, h->d_src,
-                    h->d_ctab, h->d_tbase, h->d_imask, h->d_links, h->d_amp, ap, pm, h->d_iolet_sites,
+  return launch_pdl(kernel, grid, BLOCK, st, (const S*)prev, (const S*)cur, (const S*)mu_next, (S*)mu_out, h->index(),
+                    h->d_links, h->d_amp, ap, pm, h->d_iolet_sites,
                     h->n_iolet_sites, gi, make_block_div(stride), dtau_part, dlink, st_);
 }
 

@@ -120,7 +120,7 @@ StepParams hlb_solver::params(int64_t tb) const {
 namespace {
 
 struct Layout {
-  size_t f0 = 0, f1 = 0, src = 0, ctab = 0, tbase = 0, ctflag = 0, links = 0, amp = 0, ampf = 0, normal = 0, stage = 0, red = 0, lflux = 0, isites = 0, icode = 0, imask = 0, ioff = 0,
+  size_t f0 = 0, f1 = 0, src = 0, ctab = 0, tbase = 0, rtab = 0, rbase = 0, ctflag = 0, links = 0, amp = 0, ampf = 0, normal = 0, stage = 0, red = 0, lflux = 0, isites = 0, icode = 0, imask = 0, ioff = 0,
          ilist = 0, mon = 0, wkpar = 0, wkstate = 0,
          ioval = 0, iovnext = 0, total = 0;
   int64_t n_links = 0;
@@ -240,6 +240,8 @@ Layout layout(const hlb_lattice* L, const hlb_options* o, const std::vector<int6
   y.src = off; off += align_up(sizeof(int32_t) * 18 * (size_t)row_stride(n));
   y.ctab = off; off += align_up(sizeof(uint32_t) * 9 * (size_t)row_stride(n));
   y.tbase = off; off += align_up(sizeof(int32_t) * hlb::CT_BASES * (size_t)((n + hlb::CT_TILE - 1) / hlb::CT_TILE));
+  y.rtab = off; off += align_up(sizeof(uint32_t) * hlb::CT_ROW_WORDS * (size_t)row_stride(n));
+  y.rbase = off; off += align_up(sizeof(int32_t) * hlb::CT_GROUPS * (size_t)((n + hlb::CT_TILE - 1) / hlb::CT_TILE));
   y.ctflag = off; off += align_up(sizeof(int32_t));
   y.links = off; off += align_up(sizeof(LinkRec) * (size_t)std::max<int64_t>(y.n_links, 1));
   y.amp = off; off += align_up(sizeof(double) * (size_t)std::max(y.n_groups, 1));
@@ -372,6 +374,8 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   h->d_src = (int32_t*)(base + y.src);
   h->d_ctab = (uint32_t*)(base + y.ctab);
   h->d_tbase = (int32_t*)(base + y.tbase);
+  h->d_rtab = (uint32_t*)(base + y.rtab);
+  h->d_rbase = (int32_t*)(base + y.rbase);
   int32_t* d_misfit = (int32_t*)(base + y.ctflag);
   h->d_links = (LinkRec*)(base + y.links);
   h->d_amp = (double*)(base + y.amp);

@@ -493,20 +493,54 @@ __device__ __forceinline__ const int32_t* idx_at(const int32_t* src, int i, uint
 }
 
 // ---------------------------------------------------------------------------
-// Compact index table.  The lattice is ordered lexicographically by (z, y, x)
-// and x - c_i keeps that order, so over a tile of CT_TILE consecutive sites
-// the fluid sources of one direction increase with the site index, and in
-// vessel lattices they span a few hundred sites.  Per tile and direction the
-// table keeps the smallest fluid source (tbase[tile][i - 1], CT_BASES int32
-// entries a tile, the last two unused), and per site and direction a 16-bit
-// offset from it, or CT_WALL / CT_IOLET for a link without a fluid source.
-// Directions 2p + 1 (low half) and 2p + 2 (high half) share one 32-bit word
-// in row p of ctab (rows of stride sn): 36 bytes a site instead of the 72 of
-// the 32-bit table.  A lattice with a span above CT_MAX_SPAN uses the 32-bit
-// table (the same kernels with CT = false).
+// Compact index table, one of two forms for each tile of CT_TILE sites.
+//
+// Row form.  A lattice is ordered lexicographically by (z, y, x), so the
+// sites of one lattice row (y, z) are consecutive wherever the row has no
+// hole, and the 18 sources x - c_i of a site lie in nine rows: its own, at
+// x -+ 1, and eight others, in each of which the sources of the directions
+// with the same (cy, cz) are neighbours: s = p - cx with one position p for
+// up to three directions.  p - x changes by a few sites from row to row, so
+// over a tile it fits 8 bits above the tile's smallest.  Per site three
+// 32-bit words (rows of stride sn in rtab): the bit mask of the directions
+// with a fluid source (bit i - 1; bit CT_IOLET_BIT: the site has an iolet
+// link), and the eight 8-bit offsets, group g in byte g % 4 of word 1 + g / 4.
+// Per tile the eight bases (rbase[tile][g], smallest p - x of the group).
+// 12.1 bytes a site.
+//
+// Offset form, for the tiles that a hole in a row or a wide span keeps out
+// of the row form (1.9 % of the tiles of the seeded 20M-site tree, 14 % at
+// 0.5M sites): per tile and direction the smallest fluid source
+// (tbase[tile][i - 1], CT_BASES int32 entries a tile, the last two unused),
+// and per site and direction a 16-bit offset from it, or CT_WALL / CT_IOLET
+// for a link without a fluid source.  Directions 2p + 1 (low half) and 2p + 2
+// (high half) share one 32-bit word in row p of ctab (rows of stride sn): 36
+// bytes a site.  rbase[tile][0] = CT_NO_ROWS marks such a tile.
+//
+// A lattice with a span above CT_MAX_SPAN in some tile uses the 32-bit table
+// (72 bytes a site; the same kernels with CT = false).
 // ---------------------------------------------------------------------------
 constexpr uint32_t CT_WALL = 0xffffu, CT_IOLET = 0xfffeu, CT_MAX_SPAN = 0xfffdu;
 constexpr int CT_TILE = 256, CT_BASES = 20;
+constexpr int CT_GROUPS = 8, CT_ROW_WORDS = 3, CT_IOLET_BIT = 18;
+constexpr int32_t CT_NO_ROWS = (int32_t)0x80000000;
+
+// Row-form group of direction i by (cy, cz); CT_GROUPS for the site's own row.
+__host__ __device__ constexpr int row_group(int i) {
+  return cz(i) == 0 ? (cy(i) == 0 ? CT_GROUPS : (cy(i) > 0 ? 0 : 1))
+                    : (cy(i) == 0 ? (cz(i) > 0 ? 2 : 3)
+                                  : (cz(i) > 0 ? (cy(i) > 0 ? 4 : 7) : (cy(i) > 0 ? 6 : 5)));
+}
+
+// The streaming index of a lattice as the kernels read it.
+struct IndexTables {
+  const int32_t* src;     // [18][sn] int32 codes
+  const uint32_t* ctab;   // [9][sn] offset form
+  const int32_t* tbase;   // [tiles][CT_BASES]
+  const uint32_t* rtab;   // [CT_ROW_WORDS][sn] row form
+  const int32_t* rbase;   // [tiles][CT_GROUPS]
+  const uint32_t* imask;  // [(n + 31) / 32] bit x % 32 of word x / 32: site x has an iolet link
+};
 
 // How a kernel loads its index entries: read-only cached, streaming (read
 // once, evict first), or cached in L1 for a re-read by the same thread.
@@ -516,75 +550,107 @@ __device__ __forceinline__ T ld_index(const T* p) {
   return LD == LD_STREAM ? __ldcs(p) : (LD == LD_L1 ? __ldca(p) : __ldg(p));
 }
 
-// The 18 index codes s[i - 1] of site x (tile `tile` of the compact table):
-// a fluid source's index, -1 across a wall, and for an iolet link the
-// re-coded record (32-bit table) or -2 (compact table).
-template <bool CT, bool WIDE, int LD>
-__device__ __forceinline__ void load_codes(const int32_t* __restrict__ src, const uint32_t* __restrict__ ctab,
-                                           const int32_t* __restrict__ tbase, uint32_t sn, uint32_t x,
-                                           uint32_t tile, int32_t* s) {
-  if (CT) {
-    uint32_t w[9];
+// The offset-form entries of site x: w[9] from ctab, b[i - 1] the tile's bases.
+template <bool WIDE, int LD>
+__device__ __forceinline__ void load_offset_form(const IndexTables& ix, uint32_t sn, uint32_t x, uint32_t tile,
+                                                 uint32_t* w, int32_t* b) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) w[q] = ld_index<LD>(WIDE ? ctab + ((uint64_t)q * sn + x) : ctab + (uint32_t)q * sn + x);
-    const int4* tb = reinterpret_cast<const int4*>(tbase + (uint64_t)tile * CT_BASES);
-    int b[20];
+  for (int q = 0; q < 9; ++q)
+    w[q] = ld_index<LD>(WIDE ? ix.ctab + ((uint64_t)q * sn + x) : ix.ctab + (uint32_t)q * sn + x);
+  const int4* tb = reinterpret_cast<const int4*>(ix.tbase + (uint64_t)tile * CT_BASES);
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const int4 v = __ldg(tb + q);
-      b[4 * q] = v.x;
-      b[4 * q + 1] = v.y;
-      b[4 * q + 2] = v.z;
-      b[4 * q + 3] = v.w;
-    }
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const uint32_t o = (i & 1) ? (w[(i - 1) >> 1] & 0xffffu) : (w[(i - 1) >> 1] >> 16);
-      s[i - 1] = o < CT_IOLET ? (int32_t)((uint32_t)b[i - 1] + o) : (o == CT_WALL ? -1 : -2);
-    }
-  } else {
-#pragma unroll
-    for (int i = 1; i < Q; ++i) s[i - 1] = ld_index<LD>(idx_at<WIDE>(src, i, sn, x));
+  for (int q = 0; q < 5; ++q) {
+    const int4 v = __ldg(tb + q);
+    b[4 * q] = v.x;
+    b[4 * q + 1] = v.y;
+    b[4 * q + 2] = v.z;
+    b[4 * q + 3] = v.w;
   }
 }
+// 16-bit offset of direction i among the words w[9] of a site.
+__device__ __forceinline__ uint32_t offset_of(const uint32_t* w, int i) {
+  return (i & 1) ? (w[(i - 1) >> 1] & 0xffffu) : (w[(i - 1) >> 1] >> 16);
+}
+// The tile's row-form bases; false if the tile has the offset form.
+__device__ __forceinline__ bool load_row_bases(const IndexTables& ix, uint32_t tile, int32_t* b) {
+  const int4* rb = reinterpret_cast<const int4*>(ix.rbase + (uint64_t)tile * CT_GROUPS);
+  const int4 lo = __ldg(rb), hi = __ldg(rb + 1);
+  b[0] = lo.x;
+  b[1] = lo.y;
+  b[2] = lo.z;
+  b[3] = lo.w;
+  b[4] = hi.x;
+  b[5] = hi.y;
+  b[6] = hi.z;
+  b[7] = hi.w;
+  return b[0] != CT_NO_ROWS;
+}
+// Row positions p of site x's eight groups from its two offset words; pos[8] = x.
+__device__ __forceinline__ void row_positions(uint32_t x, const int32_t* b, uint32_t w1, uint32_t w2, uint32_t* pos) {
+#pragma unroll
+  for (int g = 0; g < CT_GROUPS; ++g) pos[g] = x + (uint32_t)b[g] + (((g < 4 ? w1 : w2) >> (8 * (g & 3))) & 0xffu);
+  pos[CT_GROUPS] = x;
+}
 
-// The 18 population offsets a bulk step kernel gathers from at site x (off[i],
-// i = 1..18): for a fluid source s the slot of row i at s (pull; AAODD: row
-// opp(i) at s), otherwise row opp(i) at x itself (AAODD: row i at x), which is
-// bounce-back (iolet links get their values elsewhere).  From the compact
-// table a link is fluid exactly when its offset is below CT_IOLET, so the
-// offset goes straight into the slot without forming a signed code.
-template <bool CT, bool WIDE, int LD, bool AAODD>
-__device__ __forceinline__ void load_offsets(const int32_t* __restrict__ src, const uint32_t* __restrict__ ctab,
-                                             const int32_t* __restrict__ tbase, uint32_t sn, uint32_t n, uint32_t x,
-                                             uint32_t tile, uint32_t* off) {
+// Calls link(i, fluid, s) for the 18 directions i of site x: whether the link
+// has a fluid source, and if so its index s.  Offset form:
+template <bool WIDE, int LD, typename Link>
+__device__ __forceinline__ void offset_links(const IndexTables& ix, uint32_t sn, uint32_t x, uint32_t tile, Link&& link) {
+  uint32_t w[9];
+  int32_t b[CT_BASES];
+  load_offset_form<WIDE, LD>(ix, sn, x, tile, w, b);
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const uint32_t o = offset_of(w, i);
+    link(i, o < CT_IOLET, (uint32_t)b[i - 1] + o);
+  }
+}
+// Whichever form the tile has.  The row form costs three loads of words a site
+// and about two integer instructions a direction before the caller's select,
+// against nine loads and four instructions for the offset form.  Returns
+// whether the site has an iolet link (IOLET: asked for).
+template <bool CT, bool WIDE, int LD, bool IOLET, typename Link>
+__device__ __forceinline__ bool for_links(const IndexTables& ix, uint32_t sn, uint32_t x, uint32_t tile, Link&& link) {
   if (CT) {
-    uint32_t w[9];
+    int32_t b[CT_GROUPS];
+    if (load_row_bases(ix, tile, b)) {
+      uint32_t w[CT_ROW_WORDS], pos[CT_GROUPS + 1];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) w[q] = ld_index<LD>(WIDE ? ctab + ((uint64_t)q * sn + x) : ctab + (uint32_t)q * sn + x);
-    const int4* tb = reinterpret_cast<const int4*>(tbase + (uint64_t)tile * CT_BASES);
-    int b[20];
+      for (int q = 0; q < CT_ROW_WORDS; ++q)
+        w[q] = ld_index<LD>(WIDE ? ix.rtab + ((uint64_t)q * sn + x) : ix.rtab + (uint32_t)q * sn + x);
+      row_positions(x, b, w[1], w[2], pos);
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const int4 v = __ldg(tb + q);
-      b[4 * q] = v.x;
-      b[4 * q + 1] = v.y;
-      b[4 * q + 2] = v.z;
-      b[4 * q + 3] = v.w;
+      for (int i = 1; i < Q; ++i) link(i, (w[0] >> (i - 1)) & 1u, pos[row_group(i)] - (uint32_t)cx(i));
+      return IOLET && ((w[0] >> CT_IOLET_BIT) & 1u);
     }
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const uint32_t o = (i & 1) ? (w[(i - 1) >> 1] & 0xffffu) : (w[(i - 1) >> 1] >> 16);
-      off[i] = o < CT_IOLET ? slot<WIDE>(AAODD ? opp(i) : i, n, (uint32_t)b[i - 1] + o)
-                            : slot<WIDE>(AAODD ? i : opp(i), n, x);
-    }
+    offset_links<WIDE, LD>(ix, sn, x, tile, link);
   } else {
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-      const int32_t s = ld_index<LD>(idx_at<WIDE>(src, i, sn, x));
-      off[i] = s >= 0 ? slot<WIDE>(AAODD ? opp(i) : i, n, (uint32_t)s) : slot<WIDE>(AAODD ? i : opp(i), n, x);
+      const int32_t s = ld_index<LD>(idx_at<WIDE>(ix.src, i, sn, x));
+      link(i, s >= 0, (uint32_t)s);
     }
   }
+  return IOLET && ((__ldg(ix.imask + (x >> 5)) >> (x & 31)) & 1u);
+}
+
+// The 18 codes of site x: code[i] >= 0 is the fluid source of direction i,
+// anything negative a link without one.
+template <bool CT, bool WIDE, int LD>
+__device__ __forceinline__ void load_codes(const IndexTables& ix, uint32_t sn, uint32_t x, uint32_t tile, int32_t* code) {
+  for_links<CT, WIDE, LD, false>(ix, sn, x, tile, [&](int i, bool fluid, uint32_t s) { code[i] = fluid ? (int32_t)s : -1; });
+}
+
+// The 18 population offsets a pull step gathers from at site x (off[i], i =
+// 1..18): for a fluid source s the slot of row i at s, otherwise row opp(i) at
+// x itself, which is bounce-back (iolet links get their values elsewhere).
+// Returns whether the site has an iolet link.
+template <bool CT, bool WIDE, int LD>
+__device__ __forceinline__ bool load_offsets(const IndexTables& ix, uint32_t sn, uint32_t n, uint32_t x, uint32_t tile,
+                                             uint32_t* off) {
+  return for_links<CT, WIDE, LD, true>(ix, sn, x, tile, [&](int i, bool fluid, uint32_t s) {
+    off[i] = fluid ? slot<WIDE>(i, n, s) : slot<WIDE>(opp(i), n, x);
+  });
 }
 
 }  // namespace hlb

@@ -7,13 +7,13 @@
 // which wall links are branch-free address selects and iolet links a rare
 // per-site fix-up.  Two streaming schemes:
 //
-//  * pull A-B (k_step): read buffer A by gathering through the index table,
-//    write buffer B; 188 B per FP32 site update with the compact index
-//    table (224 B with the int32 one).
+//  * pull A-B (k_step, k_step2): read buffer A by gathering through the index
+//    table, write buffer B; 164 B per FP32 site update with the row form of
+//    the compact index table (224 B with the int32 one).
 //  * AA pattern (k_aa_even / k_aa_odd, then k_aa_fix over iolet sites): one
 //    buffer.  Even steps read a site's 19 slots and write them back swapped
 //    (no index table); odd steps read 19 slots through the index table and
-//    write the results to the very same 19 slots.  152 B (even) + 188 B
+//    write the results to the very same 19 slots.  152 B (even) + 164 B
 //    (odd; 224 B with the int32 table) per FP32 update.
 //
 // The bulk kernels take the index from its compact form (hlb_common.cuh,
@@ -35,6 +35,13 @@ using namespace hlb;
 namespace {
 
 constexpr int BLOCK = 256;
+// Two-site step kernels: threads a block (one tile), and blocks per SM.  Measured
+// on the 20M-site tree: 256 threads x 3 blocks ran the BF16 odd step in 415 us,
+// 128 x 6 in 394 (a block's slots return sooner), 128 x 7 (72 registers, a few
+// bytes of spill) in 388; FP32 532 us at 6 blocks, 539 at 7.
+constexpr int PAIR = CT_TILE / 2;
+template <typename S> constexpr int pair_blocks() { return sizeof(S) == 4 ? 6 : 7; }
+
 // Lanes a site for the iolet sites: a site's 19 directions spread over them,
 // up to ceil(19 / lanes) a lane.  Measured on the 20M-site tree: the pull
 // step's iolet sites 8 lanes (BF16 step 411 -> 405 us against 16, 418 at 32),
@@ -52,34 +59,39 @@ __device__ __forceinline__ void l2_prefetch(const void* q, uint32_t bytes) {
 
 // Called by the first warp of a bulk block: prefetch into L2 what the block
 // that takes tile `tile` (about a wave of resident blocks later) reads
-// first, so that its loads find L2 instead of waiting on DRAM.  Lanes 0-8:
-// the tile's compact index words (row q, 256 sites).  With POPS, lanes
+// first, so that its loads find L2 instead of waiting on DRAM.  Lanes 0-2:
+// the tile's row-form index words (256 sites of each).  With POPS, lanes
 // 9-26: for direction i = lane - 8, the population row its gathers read
 // (ROWOPP: row opp(i), as the AA odd step reads; else row i) from the
-// tile's base for i, 320 sites wide (the sources of a tile span about 255
-// sites on vessel lattices).  Every range is clamped to its array: ctab
-// holds 9 rows of sn words, A 19 rows of n populations.
+// tile's smallest source for i, 320 sites wide (the sources of a tile span
+// about 255 sites on vessel lattices).  A tile in offset form is left to its
+// own loads.  Every range is clamped to its array: rtab holds CT_ROW_WORDS
+// rows of sn words, A 19 rows of n populations.
 template <typename S, bool POPS, bool ROWOPP>
-__device__ __forceinline__ void prefetch_tile(const S* A, const uint32_t* __restrict__ ctab,
-                                              const int32_t* __restrict__ tbase, uint32_t n, uint32_t sn,
+__device__ __forceinline__ void prefetch_tile(const S* A, const IndexTables& ix, uint32_t n, uint32_t sn,
                                               uint32_t tile) {
   const uint32_t ntiles = (n + BLOCK - 1) / BLOCK;
   const int l = threadIdx.x & 31;
   if (tile >= ntiles) return;
   const uint64_t x0 = (uint64_t)tile * BLOCK;
-  if (l < 9) {
+  if (l < CT_ROW_WORDS) {
     const uint64_t e = x0 + BLOCK < (uint64_t)sn ? x0 + BLOCK : (uint64_t)sn;  // sn: a multiple of 4
-    l2_prefetch(ctab + (uint64_t)l * sn + x0, (uint32_t)((e - x0) * 4));
-  } else if (POPS && l < 9 + Q - 1) {
-    const int i = l - 8;
-    const uint64_t b = (uint32_t)__ldg(tbase + (uint64_t)tile * CT_BASES + (i - 1));  // < n
+    l2_prefetch(ix.rtab + (uint64_t)l * sn + x0, (uint32_t)((e - x0) * 4));
+  } else if (POPS && l >= 9 && l < 9 + Q - 1) {
+    const int i = l - 8, y = k_cy[i], z = k_cz[i];
+    const int32_t* rb = ix.rbase + (uint64_t)tile * CT_GROUPS;
+    if (__ldg(rb) == CT_NO_ROWS) return;
+    // row_group(i) of a run-time direction
+    const int g = z == 0 ? (y > 0 ? 0 : 1) : (y == 0 ? (z > 0 ? 2 : 3) : (z > 0 ? (y > 0 ? 4 : 7) : (y > 0 ? 6 : 5)));
+    const int64_t first = (int64_t)x0 - k_cx[i] + ((y | z) ? __ldg(rb + g) : 0);
+    const uint64_t b = first > 0 ? (uint64_t)first : 0;
     const uint64_t r = ROWOPP ? (uint64_t)lane_opp(i) : (uint64_t)i;
     const uint64_t e = b + 320 < (uint64_t)n ? b + 320 : (uint64_t)n;
     const uint64_t total = ((uint64_t)Q * n * sizeof(S) + 15) & ~15ull;  // within the 256-aligned section
     const uint64_t lo = ((r * n + b) * sizeof(S)) & ~15ull;
     const uint64_t hr = ((r * n + e) * sizeof(S) + 15) & ~15ull;
     const uint64_t hi = hr < total ? hr : total;
-    if (hi > lo) l2_prefetch(reinterpret_cast<const char*>(A) + lo, (uint32_t)(hi - lo));
+    if (b < (uint64_t)n && hi > lo) l2_prefetch(reinterpret_cast<const char*>(A) + lo, (uint32_t)(hi - lo));
   }
 }
 
@@ -193,42 +205,37 @@ __device__ __forceinline__ void step_iolet_site(const S* __restrict__ fin, S* __
 
 // Pull A-B step from s'(t-1) in one launch: gather f(t) through the index
 // table (walls: the site's own opposite slot), collide, store coalesced.
-// Every stride-th block (the first n_iolet_blocks of them) takes 32 iolet
+// Every stride-th block (the first n_iolet_blocks of them) takes iolet
 // sites, 8 lanes each (step_iolet_site); the others take 256 bulk sites,
 // a thread each, and leave iolet sites alone.  The iolet blocks, spread
 // through the grid, run beside the bulk blocks instead of after them.
-// WIDE: offsets within direction pairs (lattices above ~226M sites).  CT:
-// bulk codes from the compact index table (iolet warps read the 32-bit one),
-// and an L2 prefetch of the bulk tile `pf` tiles ahead, as in k_aa_odd.
+// This one-site form serves FP64 storage and the int32 table; k_step2 the
+// rest.  WIDE: offsets within direction pairs (lattices above ~226M sites).
+// CT: bulk codes from the compact index table (iolet lanes read the 32-bit
+// one), and an L2 prefetch of the bulk tile `pf` tiles ahead.
 template <typename S, bool WIDE, bool CT>
 __global__ void __launch_bounds__(BLOCK, 5) k_step(const S* __restrict__ fin, S* __restrict__ fout,
-                                                const int32_t* __restrict__ src, const uint32_t* __restrict__ ctab,
-                                                const int32_t* __restrict__ tbase, const LinkRec* __restrict__ links,
+                                                const IndexTables ix, const LinkRec* __restrict__ links,
                                                 const double* __restrict__ amp, const int32_t* __restrict__ sites,
                                                 int64_t nsites, unsigned n_iolet_blocks, const BlockDiv stride,
-                                                const uint32_t* __restrict__ imask, uint32_t pf, uint32_t tile0,
-                                                const StepParams p) {
+                                                uint32_t pf, uint32_t tile0, const StepParams p) {
   using R = typename Real<S>::type;
   const unsigned b = blockIdx.x, j = block_div(b, stride);
   if (b == j * stride.d && j < n_iolet_blocks) {
     pdl_wait();
     pdl_trigger();
-    step_iolet_site<S>(fin, fout, src, links, amp, sites, nsites, p, ((int64_t)j * BLOCK + threadIdx.x) / kStepIoletLanes);
+    step_iolet_site<S>(fin, fout, ix.src, links, amp, sites, nsites, p, ((int64_t)j * BLOCK + threadIdx.x) / kStepIoletLanes);
     return;
   }
   const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
   const uint32_t tile = tile0 + b - min(n_iolet_blocks, j + 1);
   const uint32_t x = tile * BLOCK + threadIdx.x;
-  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, false>(fin, ctab, tbase, n, sn, tile + pf);
+  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, false>(fin, ix, n, sn, tile + pf);
   uint32_t off[Q];
   const bool live = x < n;
-  // sites with an iolet link are stepped by the iolet warps (one 32-bit mask
-  // word per warp instead of a test of each of the 18 codes)
+  // sites with an iolet link are stepped by the iolet warps
   bool skip = true;
-  if (live) {
-    load_offsets<CT, WIDE, LD_STREAM, false>(src, ctab, tbase, sn, n, x, tile, off);
-    skip = (__ldg(imask + (x >> 5)) >> (x & 31)) & 1u;
-  }
+  if (live) skip = load_offsets<CT, WIDE, LD_STREAM>(ix, sn, n, x, tile, off);
   pdl_wait();
   pdl_trigger();
   if (skip) return;
@@ -406,79 +413,102 @@ __device__ __forceinline__ void collide_pair(const float2* h, float omega, Emit&
   }
 }
 
-// Pull A-B step (k_step) with two neighbouring sites x, x + 1 per thread (n
-// even, compact table, 32-bit offsets; FP32 or 16-bit storage): the index
-// words of both in one 8-byte load per row, the two collisions in paired
-// FP32 instructions (collide_pair: the bits of k_step) and one store of the
-// pair per direction; the gathers stay one per site and direction.  A block
-// takes two tiles.  A pair with one iolet site stores only its other site.
-// Three blocks per SM (80 registers), on the 20M-site tree: BF16 447 -> 419
-// us (four blocks, 64 registers with spills: 485 us), FP32 577 -> 567 us.
-// The same pairing in the AA odd step, whose stores scatter, was slower
-// (463 -> 563 us BF16).
-template <typename S>
-__global__ void __launch_bounds__(BLOCK, 3) k_step2(const S* __restrict__ fin, S* __restrict__ fout,
-                                                 const int32_t* __restrict__ src, const uint32_t* __restrict__ ctab,
-                                                 const int32_t* __restrict__ tbase, const LinkRec* __restrict__ links,
-                                                 const double* __restrict__ amp, const int32_t* __restrict__ sites,
-                                                 int64_t nsites, unsigned n_iolet_blocks, const BlockDiv stride,
-                                                 const uint32_t* __restrict__ imask, uint32_t pf,
-                                                 const StepParams p) {
-  using P = Pair<S>;
-  using T = typename P::T;
+// Two sites a thread on the compact table (k_step2, k_aa_odd2): thread t of a
+// block takes sites x = 64 (t / 32) + t % 32 and x + 32 of the block's tile, so
+// every load and store of a warp stays one run of 32 sites.
+__device__ __forceinline__ uint32_t pair_site(uint32_t tile) {
+  return tile * CT_TILE + 2 * (threadIdx.x & ~31u) + (threadIdx.x & 31u);
+}
+// Row-form words of the pair's sites (y = x + 32 may lie past the end: x's then).
+__device__ __forceinline__ void load_pair_words(const IndexTables& ix, bool wide, uint32_t sn, uint32_t x, uint32_t y,
+                                                uint32_t* wa, uint32_t* wb) {
+#pragma unroll
+  for (int q = 0; q < CT_ROW_WORDS; ++q) {
+    const uint32_t* row = wide ? ix.rtab + (uint64_t)q * sn : ix.rtab + (uint32_t)q * sn;
+    wa[q] = __ldg(row + x);
+    wb[q] = __ldg(row + y);
+  }
+}
+// Offset that direction i of site x is read from (pull), or read from and
+// written to (AAODD), given its row-form mask and positions.
+template <bool WIDE, bool AAODD>
+__device__ __forceinline__ uint32_t row_offset(int i, uint32_t mask, const uint32_t* pos, uint32_t n) {
+  const uint32_t s = pos[row_group(i)] - (uint32_t)cx(i);
+  return ((mask >> (i - 1)) & 1u) ? slot<WIDE>(AAODD ? opp(i) : i, n, s) : slot<WIDE>(AAODD ? i : opp(i), n, pos[CT_GROUPS]);
+}
+
+// Pull A-B step (k_step) with two sites a thread, FP32 or 16-bit storage on the
+// compact table, any number of sites.  Bound by DRAM in FP32 (164 bytes a
+// site with the row-form index) and by instruction issue and latency in 16
+// bits.  Pairing halves the arithmetic: the two collisions run in paired FP32
+// instructions (collide_pair: the bits of k_step).  The pair is x and x + 32,
+// not two neighbours: a warp's gather of neighbours spans 64 sites in steps
+// of two, twice the sectors a request, and needs an even site count for its
+// vector stores.  20M-site tree, per step: FP32 563 -> 495 us, BF16 406 -> 345
+// us against neighbours on the 16-bit offset table; 2.0M sites (odd) FP32 66.5
+// -> 56.4 us, BF16 47.7 -> 38.7 us against one site a thread on it.
+// Prefetch 3 tiles per SM ahead: FP32 495 us with the gathered rows, 500
+// without them, 516 with no prefetch, 537 at 6; 16-bit storage prefetches
+// the index words only.  A tile in offset form takes its sites one by one.
+template <typename S, bool WIDE>
+__global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_step2(const S* __restrict__ fin, S* __restrict__ fout,
+                                                const IndexTables ix, const LinkRec* __restrict__ links,
+                                                const double* __restrict__ amp, const int32_t* __restrict__ sites,
+                                                int64_t nsites, unsigned n_iolet_blocks, const BlockDiv stride,
+                                                uint32_t pf, uint32_t tile0, const StepParams p) {
   const unsigned b = blockIdx.x, j = block_div(b, stride);
   if (b == j * stride.d && j < n_iolet_blocks) {
     pdl_wait();
     pdl_trigger();
-    step_iolet_site<S>(fin, fout, src, links, amp, sites, nsites, p, ((int64_t)j * BLOCK + threadIdx.x) / kStepIoletLanes);
+    step_iolet_site<S>(fin, fout, ix.src, links, amp, sites, nsites, p, ((int64_t)j * PAIR + threadIdx.x) / kStepIoletLanes);
     return;
   }
   const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
-  const uint32_t k = b - min(n_iolet_blocks, j + 1);  // bulk block: tiles 2k, 2k + 1
-  const uint32_t x = 2 * (k * BLOCK + threadIdx.x);
-  const uint32_t tile = x / CT_TILE;
-  if (pf && threadIdx.x < 64) prefetch_tile<S, false, false>(fin, ctab, tbase, n, sn, 2 * (k + pf) + (threadIdx.x >> 5));
-  uint32_t m = 3u;  // bit 0: x is stepped elsewhere (iolet warps, or x >= n), bit 1: x + 1
-  uint32_t off[2][Q];
-  if (x < n) {
-    m = (__ldg(imask + (x >> 5)) >> (x & 31)) & 3u;  // x even: both bits in one word
-    uint2 w[9];
+  const uint32_t tile = tile0 + b - min(n_iolet_blocks, j + 1);
+  const uint32_t x = pair_site(tile), y = x + 32;
+  if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, false>(fin, ix, n, sn, tile + pf);
+  int32_t bs[CT_GROUPS];
+  if (load_row_bases(ix, tile, bs)) {
+    const uint32_t y1 = y < n ? y : x;  // a thread without a second site repeats its first, and does not store it
+    uint32_t wa[CT_ROW_WORDS], wb[CT_ROW_WORDS];
+    if (x < n) load_pair_words(ix, WIDE, sn, x, y1, wa, wb);
+    pdl_wait();
+    pdl_trigger();
+    if (x >= n) return;
+    const bool da = !((wa[0] >> CT_IOLET_BIT) & 1u), db = y < n && !((wb[0] >> CT_IOLET_BIT) & 1u);
+    uint32_t pa[CT_GROUPS + 1], pb[CT_GROUPS + 1];
+    row_positions(x, bs, wa[1], wa[2], pa);
+    row_positions(y1, bs, wb[1], wb[2], pb);
+    float2 h[Q];
+    h[0] = make_float2(ldpop(fin + x), ldpop(fin + y1));
 #pragma unroll
-    for (int q = 0; q < 9; ++q) w[q] = __ldcs(reinterpret_cast<const uint2*>(ctab + (uint32_t)q * sn + x));
-    const int4* tb = reinterpret_cast<const int4*>(tbase + (uint64_t)tile * CT_BASES);
-    int bs[20];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const int4 v = __ldg(tb + q);
-      bs[4 * q] = v.x;
-      bs[4 * q + 1] = v.y;
-      bs[4 * q + 2] = v.z;
-      bs[4 * q + 3] = v.w;
-    }
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const uint32_t wa = w[(i - 1) >> 1].x, wb = w[(i - 1) >> 1].y;
-      const uint32_t oa = (i & 1) ? (wa & 0xffffu) : (wa >> 16), ob = (i & 1) ? (wb & 0xffffu) : (wb >> 16);
-      off[0][i] = oa < CT_IOLET ? (uint32_t)i * n + (uint32_t)bs[i - 1] + oa : (uint32_t)opp(i) * n + x;
-      off[1][i] = ob < CT_IOLET ? (uint32_t)i * n + (uint32_t)bs[i - 1] + ob : (uint32_t)opp(i) * n + x + 1;
-    }
+    for (int i = 1; i < Q; ++i)
+      h[i] = make_float2(ldpop(at<WIDE>(fin, i, n, row_offset<WIDE, false>(i, wa[0], pa, n))),
+                         ldpop(at<WIDE>(fin, i, n, row_offset<WIDE, false>(i, wb[0], pb, n))));
+    collide_pair(h, p.omegaf, [&](int i, float2 v) {
+      S* o = i == 0 ? fout + x : at<WIDE>(fout, i, n, slot<WIDE>(i, n, x));
+      if (da) stpop<S>(o, v.x);
+      if (db) stpop<S>(o + 32, v.y);
+    });
+    return;
   }
-  pdl_wait();
+  for (uint32_t z = x; z < n && z <= y; z += 32) {
+    uint32_t off[Q];
+    offset_links<WIDE, LD_NC>(ix, sn, z, tile, [&](int i, bool fluid, uint32_t s) {
+      off[i] = fluid ? slot<WIDE>(i, n, s) : slot<WIDE>(opp(i), n, z);
+    });
+    pdl_wait();
+    if ((__ldg(ix.imask + (z >> 5)) >> (z & 31)) & 1u) continue;
+    float h[Q];
+    h[0] = ldpop(fin + z);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) h[i] = ldpop(at<WIDE>(fin, i, n, off[i]));
+    collide<float>(h, p.omegaf);
+    stpop<S>(fout + z, h[0]);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) stpop<S>(at<WIDE>(fout, i, n, slot<WIDE>(i, n, z)), h[i]);
+  }
   pdl_trigger();
-  if (m == 3u) return;
-  const T* fin2 = reinterpret_cast<const T*>(fin);
-  float2 h[Q];
-  h[0] = P::to(__ldg(fin2 + x / 2));
-#pragma unroll
-  for (int i = 1; i < Q; ++i) h[i] = make_float2(ldpop(fin + off[0][i]), ldpop(fin + off[1][i]));
-  if (m == 0u) {
-    T* fout2 = reinterpret_cast<T*>(fout);
-    collide_pair(h, p.omegaf, [&](int i, float2 v) { __stcs(fout2 + ((uint32_t)i * n + x) / 2, P::from(v.x, v.y)); });
-  } else {
-    const uint32_t y = m == 1u ? x + 1 : x;  // the pair's site without iolet links
-    collide_pair(h, p.omegaf,
-                 [&](int i, float2 v) { stpop<S>(fout + (uint32_t)i * n + y, m == 1u ? v.y : v.x); });
-  }
 }
 
 // Boundary value of iolet link (pull direction i, record L) at a site whose
@@ -584,28 +614,21 @@ __global__ void __launch_bounds__(256, 8) k_aa_fix(S* A, const int32_t* __restri
 // post-collision population into the slot it came from, where the site
 // downstream (or, across a wall or iolet, the site itself) reads it in the
 // next (even) step.  Iolet links get their boundary values from k_aa_fix.
-// The 18 slot offsets (32-bit) are computed once and held in registers for
-// the stores, so the index row is read once.  Five resident blocks per SM
-// (48 registers, a few bytes of spill in FP32) measured fastest.  WIDE:
-// offsets within direction pairs (lattices above ~226M sites), which need a
-// few more registers: four blocks per SM (64 registers) measured 8 % faster
-// than five with their spills.  CT: codes from the compact index table, and
-// the first warp prefetches into L2 the tile `pf` blocks ahead (0: none):
-// index words, and for 4- and 8-byte storage the gathered rows (for 16-bit
-// storage the rows measured slower).  With 32-bit offsets pf is 3 blocks per
-// SM, 0.6 of a wave: FP32 odd step 608 us at one wave, 599 us at 0.6, 615 us
-// at 0.2 (16-bit unchanged); the wide form keeps one wave (4 blocks per SM).
+// This one-site form serves FP64 storage and the int32 table; k_aa_odd2 the
+// rest.  The 18 slot offsets (32-bit) are computed once and held in registers
+// for the stores, so the index row is read once.  WIDE: offsets within
+// direction pairs (lattices above ~226M sites), four blocks per SM instead
+// of five.  CT: codes from the compact index table, and the first warp
+// prefetches into L2 the tile `pf` blocks ahead (0: none).
 template <typename S, bool WIDE, bool CT>
-__global__ void __launch_bounds__(BLOCK, WIDE ? 4 : 5) k_aa_odd(S* A, const int32_t* __restrict__ src,
-                                                               const uint32_t* __restrict__ ctab,
-                                                               const int32_t* __restrict__ tbase, uint32_t pf,
+__global__ void __launch_bounds__(BLOCK, WIDE ? 4 : 5) k_aa_odd(S* A, const IndexTables ix, uint32_t pf,
                                                                const StepParams p) {
   using R = typename Real<S>::type;
   const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
   const uint32_t x = blockIdx.x * BLOCK + threadIdx.x;
-  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, true>(A, ctab, tbase, n, sn, blockIdx.x + pf);
-  int32_t code[Q - 1];
-  if (x < n) load_codes<CT, WIDE, LD_NC>(src, ctab, tbase, sn, x, blockIdx.x, code);
+  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, true>(A, ix, n, sn, blockIdx.x + pf);
+  int32_t code[Q];
+  if (x < n) load_codes<CT, WIDE, LD_NC>(ix, sn, x, blockIdx.x, code);
   pdl_wait();
   pdl_trigger();
   if (x >= n) return;
@@ -614,9 +637,8 @@ __global__ void __launch_bounds__(BLOCK, WIDE ? 4 : 5) k_aa_odd(S* A, const int3
   h[0] = to_real(A[x]);
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
-    const int32_t s = code[i - 1];
     // slot opp(i) of the source, or slot i of x itself across a wall or iolet
-    off[i] = s >= 0 ? slot<WIDE>(opp(i), n, (uint32_t)s) : slot<WIDE>(i, n, x);
+    off[i] = code[i] >= 0 ? slot<WIDE>(opp(i), n, (uint32_t)code[i]) : slot<WIDE>(i, n, x);
     h[i] = to_real(*at<WIDE>(A, i, n, off[i]));
   }
   collide<R>(h, omega_of<R>(p));
@@ -625,25 +647,161 @@ __global__ void __launch_bounds__(BLOCK, WIDE ? 4 : 5) k_aa_odd(S* A, const int3
   for (int i = 1; i < Q; ++i) stpop<S>(at<WIDE>(A, i, n, off[i]), h[opp(i)]);
 }
 
+// The odd step with two sites a thread (k_step2's pairing: x and x + 32), FP32 or
+// 16-bit storage on the compact table.  A site's offsets follow from three
+// index words, so they are formed twice, for the gather and for the stores,
+// instead of being held across the collision in 36 registers: that is what
+// lets two sites share a thread at 80 (72) registers.  20M-site tree, step
+// with the iolet pass: FP32 597 -> 532 us, BF16 460 -> 388 us; 2.0M sites FP32
+// 75 -> 67, BF16 58 -> 48 us.
+template <typename S, bool WIDE>
+__global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_aa_odd2(S* A, const IndexTables ix, uint32_t pf,
+                                                               const StepParams p) {
+  const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn, tile = blockIdx.x;
+  const uint32_t x = pair_site(tile), y = x + 32;
+  if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, true>(A, ix, n, sn, tile + pf);
+  int32_t bs[CT_GROUPS];
+  if (load_row_bases(ix, tile, bs)) {
+    const bool two = y < n;
+    const uint32_t y1 = two ? y : x;  // a thread without a second site repeats its first, and does not store it
+    uint32_t wa[CT_ROW_WORDS], wb[CT_ROW_WORDS];
+    if (x < n) load_pair_words(ix, WIDE, sn, x, y1, wa, wb);
+    pdl_wait();
+    pdl_trigger();
+    if (x >= n) return;
+    uint32_t pa[CT_GROUPS + 1], pb[CT_GROUPS + 1];
+    row_positions(x, bs, wa[1], wa[2], pa);
+    row_positions(y1, bs, wb[1], wb[2], pb);
+    float2 h[Q];
+    h[0] = make_float2(to_real(A[x]), to_real(A[y1]));
+#pragma unroll
+    for (int i = 1; i < Q; ++i)
+      h[i] = make_float2(to_real(*at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wa[0], pa, n))),
+                         to_real(*at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wb[0], pb, n))));
+    float2 o[Q];
+    collide_pair(h, p.omegaf, [&](int i, float2 v) { o[i] = v; });
+    // the offsets again, from the words: held across the collision they would cost 36 registers
+#pragma unroll
+    for (int q = 0; q < CT_ROW_WORDS; ++q) asm volatile("" : "+r"(wa[q]), "+r"(wb[q]));
+    load_row_bases(ix, tile, bs);
+    row_positions(x, bs, wa[1], wa[2], pa);
+    row_positions(y, bs, wb[1], wb[2], pb);
+    stpop<S>(A + x, o[0].x);
+    if (two) stpop<S>(A + y, o[0].y);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      stpop<S>(at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wa[0], pa, n)), o[opp(i)].x);
+      if (two) stpop<S>(at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wb[0], pb, n)), o[opp(i)].y);
+    }
+    return;
+  }
+  pdl_wait();
+  pdl_trigger();
+  for (uint32_t z = x; z < n && z <= y; z += 32) {
+    int32_t code[Q];
+    offset_links<WIDE, LD_NC>(ix, sn, z, tile, [&](int i, bool fluid, uint32_t s) { code[i] = fluid ? (int32_t)s : -1; });
+    uint32_t off[Q];
+    float h[Q];
+    h[0] = to_real(A[z]);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      off[i] = code[i] >= 0 ? slot<WIDE>(opp(i), n, (uint32_t)code[i]) : slot<WIDE>(i, n, z);
+      h[i] = to_real(*at<WIDE>(A, i, n, off[i]));
+    }
+    collide<float>(h, p.omegaf);
+    stpop<S>(A + z, h[0]);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) stpop<S>(at<WIDE>(A, i, n, off[i]), h[opp(i)]);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Compact index table (layout in hlb_common.cuh), built once from the 32-bit
-// table: one block per tile.  Per direction the block finds the smallest and
-// largest fluid source of its sites (warp min/max, then across the eight
-// warps), writes the base, and each thread its offset; pairs of directions
-// share a word.  Padding entries (n <= x < sn) read as walls.
+// table: one block per tile.  A thread loads its site's 18 codes, and the
+// block finds whether the row form holds for all of its sites (a source of
+// the own row at x - cx, one position a group, spans of 8 bits) and the
+// groups' bases.  Otherwise the block writes the offset form: per direction
+// the smallest and largest fluid source (warp min/max, then across the eight
+// warps), the base, and each thread its offset; pairs of directions share a
+// word.  Padding entries (n <= x < sn) read as walls.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(CT_TILE) k_ctab_build(const int32_t* __restrict__ src, int64_t n, int64_t sn,
                                                         uint32_t* __restrict__ ctab, int32_t* __restrict__ tbase,
+                                                        uint32_t* __restrict__ rtab, int32_t* __restrict__ rbase,
                                                         int32_t* __restrict__ misfit) {
   static_assert(CT_TILE == 256, "eight warps a tile");
   __shared__ uint32_t smin[8], smax[8];
+  __shared__ int32_t gmin[8][CT_GROUPS], gmax[8][CT_GROUPS];
   const int64_t x = (int64_t)blockIdx.x * CT_TILE + threadIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t word = 0;
+  int32_t s[Q];
+#pragma unroll
+  for (int i = 1; i < Q; ++i) s[i] = x < n ? src[(int64_t)(i - 1) * sn + x] : -1;
+  // row form: per group the position p = s + cx less x
+  constexpr int32_t NONE = INT32_MAX;
+  uint32_t mask = 0;
+  int32_t d[CT_GROUPS];
+#pragma unroll
+  for (int g = 0; g < CT_GROUPS; ++g) d[g] = NONE;
+  bool rows = true;
+#pragma unroll
   for (int i = 1; i < Q; ++i) {
-    const int32_t s = x < n ? src[(int64_t)(i - 1) * sn + x] : -1;
-    uint32_t lo = __reduce_min_sync(0xffffffffu, s >= 0 ? (uint32_t)s : 0xffffffffu);
-    uint32_t hi = __reduce_max_sync(0xffffffffu, s >= 0 ? (uint32_t)s : 0u);
+    if (s[i] <= -2) mask |= 1u << CT_IOLET_BIT;
+    if (s[i] < 0) continue;
+    mask |= 1u << (i - 1);
+    const int32_t v = (int32_t)((int64_t)s[i] + cx(i) - x);
+    const int g = row_group(i);
+    if (g == CT_GROUPS) {
+      rows &= v == 0;
+    } else {
+      rows &= d[g] == NONE || d[g] == v;
+      d[g] = v;
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < CT_GROUPS; ++g) {
+    const int32_t lo = __reduce_min_sync(FULL_MASK, d[g]), hi = __reduce_max_sync(FULL_MASK, d[g] == NONE ? INT32_MIN : d[g]);
+    if (lane == 0) {
+      gmin[wid][g] = lo;
+      gmax[wid][g] = hi;
+    }
+  }
+  rows = __syncthreads_and(rows);
+  int32_t base[CT_GROUPS];
+#pragma unroll
+  for (int g = 0; g < CT_GROUPS; ++g) {
+    int32_t lo = gmin[0][g], hi = gmax[0][g];
+    for (int k = 1; k < 8; ++k) {
+      lo = min(lo, gmin[k][g]);
+      hi = max(hi, gmax[k][g]);
+    }
+    base[g] = lo == NONE ? 0 : lo;  // no site of the tile has a fluid source in the group
+    rows &= lo == NONE || (int64_t)hi - lo <= 255;
+  }
+  if (threadIdx.x < CT_GROUPS) {
+    int32_t v = CT_NO_ROWS;
+#pragma unroll
+    for (int g = 0; g < CT_GROUPS; ++g)
+      if (rows && (int)threadIdx.x == g) v = base[g];
+    rbase[(int64_t)blockIdx.x * CT_GROUPS + threadIdx.x] = v;
+  }
+  if (rows) {  // uniform over the block
+    uint32_t w[2] = {0u, 0u};
+#pragma unroll
+    for (int g = 0; g < CT_GROUPS; ++g)
+      if (d[g] != NONE) w[g / 4] |= (uint32_t)(d[g] - base[g]) << (8 * (g % 4));
+    if (x < sn) {
+      rtab[x] = mask;
+      rtab[sn + x] = w[0];
+      rtab[2 * sn + x] = w[1];
+    }
+    return;
+  }
+  uint32_t word = 0;
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    uint32_t lo = __reduce_min_sync(FULL_MASK, s[i] >= 0 ? (uint32_t)s[i] : 0xffffffffu);
+    uint32_t hi = __reduce_max_sync(FULL_MASK, s[i] >= 0 ? (uint32_t)s[i] : 0u);
     if (lane == 0) {
       smin[wid] = lo;
       smax[wid] = hi;
@@ -657,12 +815,12 @@ __global__ void __launch_bounds__(CT_TILE) k_ctab_build(const int32_t* __restric
     }
     __syncthreads();
     const bool any = lo != 0xffffffffu;  // some site of the tile has a fluid source
-    const uint32_t base = any ? lo : 0u;
+    const uint32_t b = any ? lo : 0u;
     if (threadIdx.x == 0) {
-      tbase[(int64_t)blockIdx.x * CT_BASES + (i - 1)] = (int32_t)base;
+      tbase[(int64_t)blockIdx.x * CT_BASES + (i - 1)] = (int32_t)b;
       if (any && hi - lo > CT_MAX_SPAN) atomicOr(misfit, 1);
     }
-    const uint32_t o = s >= 0 ? ((uint32_t)s - base) & 0xffffu : (s == -1 ? CT_WALL : CT_IOLET);
+    const uint32_t o = s[i] >= 0 ? ((uint32_t)s[i] - b) & 0xffffu : (s[i] == -1 ? CT_WALL : CT_IOLET);
     if (i & 1) {
       word = o;
     } else {
@@ -909,22 +1067,24 @@ cudaError_t dispatch(int precision, A... a) {
 template <typename S>
 cudaError_t launch_gather(const hlb_solver* h, const void* fin, void* fout, const StepParams& p, uint32_t tile0,
                           uint32_t ntiles, bool iolets, cudaStream_t s) {
-  constexpr unsigned per_block = BLOCK / kStepIoletLanes;  // iolet sites a block
-  const unsigned gi = iolets ? (unsigned)((h->n_iolet_sites + per_block - 1) / per_block) : 0u;
-  const unsigned grid = gi + ntiles;
-  if (grid == 0) return cudaSuccess;
   if constexpr (sizeof(S) <= 4) {
-    if (h->compact && h->off32 && h->n % 2 == 0 && tile0 == 0 && ntiles == grid_for(h->n)) {
-      const unsigned g2 = gi + (unsigned)((h->n + 2 * BLOCK - 1) / (2 * BLOCK));
-      return launch_pdl(k_step2<S>, g2, BLOCK, s, (const S*)fin, (S*)fout, h->d_src, h->d_ctab, h->d_tbase,
-                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, gi,
-                        make_block_div(gi ? g2 / gi : 1), h->d_imask, (uint32_t)h->n_sm * 3u, p);
+    if (h->compact) {
+      const unsigned gi = iolets ? (unsigned)((h->n_iolet_sites * kStepIoletLanes + PAIR - 1) / PAIR) : 0u;
+      const unsigned grid = gi + ntiles;
+      if (grid == 0) return cudaSuccess;
+      return launch_pdl(h->off32 ? k_step2<S, false> : k_step2<S, true>, grid, PAIR, s, (const S*)fin, (S*)fout, h->index(),
+                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, gi, make_block_div(gi ? grid / gi : 1),
+                        (uint32_t)h->n_sm * 3u, tile0, p);
     }
   }
-  auto kernel = h->compact ? (h->off32 ? k_step<S, false, true> : k_step<S, true, true>)
+  const unsigned gi = iolets ? (unsigned)((h->n_iolet_sites * kStepIoletLanes + BLOCK - 1) / BLOCK) : 0u;
+  const unsigned grid = gi + ntiles;
+  if (grid == 0) return cudaSuccess;
+  constexpr bool CT = sizeof(S) > 4;  // FP64 only: the others take two sites a thread
+  auto kernel = h->compact ? (h->off32 ? k_step<S, false, CT> : k_step<S, true, CT>)
                            : (h->off32 ? k_step<S, false, false> : k_step<S, true, false>);
-  return launch_pdl(kernel, grid, BLOCK, s, (const S*)fin, (S*)fout, h->d_src, h->d_ctab, h->d_tbase, h->d_links,
-                    h->d_amp, h->d_iolet_sites, h->n_iolet_sites, gi, make_block_div(gi ? grid / gi : 1), h->d_imask,
+  return launch_pdl(kernel, grid, BLOCK, s, (const S*)fin, (S*)fout, h->index(), h->d_links, h->d_amp,
+                    h->d_iolet_sites, h->n_iolet_sites, gi, make_block_div(gi ? grid / gi : 1),
                     (uint32_t)h->n_sm * 5u, tile0, p);
 }
 
@@ -966,15 +1126,25 @@ cudaError_t aa_even<__half>(const hlb_solver* h, __half* A, const StepParams& p,
 }
 
 template <typename S>
+cudaError_t aa_odd(const hlb_solver* h, S* A, const StepParams& p, cudaStream_t s) {
+  if constexpr (sizeof(S) <= 4) {
+    if (h->compact)
+      return launch_pdl(h->off32 ? k_aa_odd2<S, false> : k_aa_odd2<S, true>, grid_for(h->n), PAIR, s, A, h->index(),
+                        (uint32_t)h->n_sm * 3u, p);
+  }
+  constexpr bool CT = sizeof(S) > 4;  // FP64 only: the others take two sites a thread
+  return launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, CT> : k_aa_odd<S, true, CT>)
+                               : (h->off32 ? k_aa_odd<S, false, false> : k_aa_odd<S, true, false>),
+                    grid_for(h->n), BLOCK, s, A, h->index(), (uint32_t)h->n_sm * (h->off32 ? 3u : 4u), p);
+}
+
+template <typename S>
 struct AAOp {
   static cudaError_t run(const hlb_solver* h, void* A, bool odd, int64_t t, cudaStream_t s) {
     StepParams p = h->params(t);
     cudaError_t e;
     if (odd)
-      e = launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, true> : k_aa_odd<S, true, true>)
-                                : (h->off32 ? k_aa_odd<S, false, false> : k_aa_odd<S, true, false>),
-                     grid_for(h->n), BLOCK, s, (S*)A, h->d_src, h->d_ctab, h->d_tbase,
-                     (uint32_t)h->n_sm * (h->off32 ? 3u : 4u), p);
+      e = aa_odd<S>(h, (S*)A, p, s);
     else
       e = aa_even<S>(h, (S*)A, p, s);
     if (e != cudaSuccess || h->n_iolet_sites == 0) return e;
@@ -1235,7 +1405,8 @@ cudaError_t hlb_launch_state(const hlb_solver* h, const void* fin, int mode, int
 }
 cudaError_t hlb_launch_ctab(const hlb_solver* h, int32_t* misfit, cudaStream_t s) {
   const int64_t tiles = (h->sn + CT_TILE - 1) / CT_TILE;
-  k_ctab_build<<<(unsigned)tiles, CT_TILE, 0, s>>>(h->d_src, h->n, h->sn, h->d_ctab, h->d_tbase, misfit);
+  k_ctab_build<<<(unsigned)tiles, CT_TILE, 0, s>>>(h->d_src, h->n, h->sn, h->d_ctab, h->d_tbase, h->d_rtab,
+                                                        h->d_rbase, misfit);
   return cudaGetLastError();
 }
 cudaError_t hlb_launch_init(const hlb_solver* h, void* f, double rho0, const float* u0, cudaStream_t s) {

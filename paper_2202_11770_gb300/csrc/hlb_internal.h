@@ -60,8 +60,12 @@ struct hlb_solver {
 
   // device tables (inside the caller's workspace)
   int32_t* d_src = nullptr;           // [18][n], iolet links re-coded to -(2 + record)
-  uint32_t* d_ctab = nullptr;         // compact index table [9][sn] (hlb_common.cuh)
-  int32_t* d_tbase = nullptr;         // its per-tile bases [tiles][CT_BASES]
+  // compact index table (hlb_common.cuh): offset form [9][sn] with its bases
+  // [tiles][CT_BASES], row form [CT_ROW_WORDS][sn] with its bases [tiles][CT_GROUPS]
+  uint32_t* d_ctab = nullptr;
+  int32_t* d_tbase = nullptr;
+  uint32_t* d_rtab = nullptr;
+  int32_t* d_rbase = nullptr;
   bool compact = false;               // bulk step and adjoint codes from the compact table
   hlb::LinkRec* d_links = nullptr;
   double* d_amp = nullptr;            // [n_groups_total]
@@ -91,6 +95,7 @@ struct hlb_solver {
   int64_t n_iolet_sites = 0;
   int64_t red_slots = 0;
 
+  hlb::IndexTables index() const { return {d_src, d_ctab, d_tbase, d_rtab, d_rbase, d_imask}; }
   size_t elem_bytes() const;
   size_t state_bytes() const { return elem_bytes() * 19 * (size_t)n; }
   // kernel parameters for a launch that gathers with boundary data at time tb
