@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(BLOCK, sizeof(typename Real<S>::type) == 8 ? 2
 // mu(N) = dJ/df(N), dJ/df_j = (2/N) (u.axis - target) (c_j.axis - u.axis) / rho
 // (added to mu, which holds zeros).
 template <typename S, int MODE>
-__global__ void k_probe_adj(const S* __restrict__ fin, const int32_t* __restrict__ src,
+__global__ void k_probe_adj(const S* __restrict__ fin, const IndexTables ix,
                             const LinkRec* __restrict__ links, const double* __restrict__ amp, const StepParams p,
                             const int64_t* __restrict__ sites, const double* __restrict__ target, double ax,
                             double ay, double az, double invN, int64_t np, S* __restrict__ mu,
@@ -466,7 +466,7 @@ __global__ void k_probe_adj(const S* __restrict__ fin, const int32_t* __restrict
   if (q >= np) return;
   const int64_t x = sites[q];
   R h[Q];
-  load_state<S, MODE>(fin, src, links, amp, p, x, h);
+  load_state<S, MODE, false, false>(fin, ix, links, amp, p, x, 0u, h);
   const Macro<R> m = moments<R>(h);
   const double uad = (double)m.ux * ax + (double)m.uy * ay + (double)m.uz * az;
   const double dd = uad - target[q];
@@ -546,7 +546,7 @@ cudaError_t launch_probe_adj(const hlb_solver* h, const void* fin, int mode, int
   if (pr.np == 0) return cudaSuccess;
   StepParams p = h->params(tb);
   const unsigned g = (unsigned)((pr.np + 127) / 128);
-  PROBE_MODE_SWITCH(mode, (k_probe_adj<S, M><<<g, 128, 0, st>>>((const S*)fin, h->d_src, h->d_links, h->d_amp, p,
+  PROBE_MODE_SWITCH(mode, (k_probe_adj<S, M><<<g, 128, 0, st>>>((const S*)fin, h->index(), h->d_links, h->d_amp, p,
                                                                  pr.sites, pr.target, pr.ax, pr.ay, pr.az, pr.invN,
                                                                  pr.np, (S*)mu, jp)));
   return cudaGetLastError();

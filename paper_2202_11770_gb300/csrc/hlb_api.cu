@@ -121,7 +121,7 @@ namespace {
 
 struct Layout {
   size_t f0 = 0, f1 = 0, src = 0, ctab = 0, tbase = 0, rtab = 0, rbase = 0, ctflag = 0, links = 0, amp = 0, ampf = 0, normal = 0, stage = 0, red = 0, lflux = 0, isites = 0, icode = 0, imask = 0, ioff = 0,
-         ilist = 0, mon = 0, wkpar = 0, wkstate = 0,
+         ilist = 0, msite = 0, mon = 0, wkpar = 0, wkstate = 0,
          ioval = 0, iovnext = 0, total = 0;
   int64_t n_links = 0;
   int32_t n_groups = 0;
@@ -255,6 +255,7 @@ Layout layout(const hlb_lattice* L, const hlb_options* o, const std::vector<int6
   y.imask = off; off += align_up(sizeof(uint32_t) * (size_t)((n + 31) / 32));
   y.ioff = off; off += align_up(sizeof(int64_t) * (size_t)(L->n_iolets + 1));
   y.ilist = off; off += align_up(sizeof(int32_t) * (size_t)std::max<int64_t>(y.n_links, 1));  // >= sites per iolet
+  y.msite = off; off += align_up(sizeof(double) * 2 * (size_t)std::max<int64_t>(y.n_links, 1));
   y.mon = off; off += align_up(sizeof(double) * 2 * (size_t)std::max(L->n_iolets, 1));
   y.wkpar = off; off += align_up(sizeof(double) * 4 * (size_t)std::max(L->n_iolets, 1));
   y.wkstate = off; off += align_up(sizeof(double) * 2 * (size_t)std::max(L->n_iolets, 1));
@@ -390,6 +391,7 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   h->d_imask = (uint32_t*)(base + y.imask);
   h->d_ioff = (int64_t*)(base + y.ioff);
   h->d_ilist = (int32_t*)(base + y.ilist);
+  h->d_msite = (double*)(base + y.msite);
   h->d_mon = (double*)(base + y.mon);
   h->d_wkpar = (double*)(base + y.wkpar);
   h->d_wkstate = (double*)(base + y.wkstate);
@@ -526,6 +528,7 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
     ilist.insert(ilist.end(), per_io[(size_t)k].begin(), per_io[(size_t)k].end());
     ioff[(size_t)k + 1] = (int64_t)ilist.size();
   }
+  h->n_ilist = (int64_t)ilist.size();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->d_ioff, ioff.data(), sizeof(int64_t) * ioff.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !ilist.empty())
@@ -723,43 +726,47 @@ extern "C" int hlb_read_macros(hlb_solver* h, float* rho, float* u, float* wss, 
   return HLB_OK;
 }
 
-static int hlb_reduce_impl(hlb_solver* h, double* mass, double* flux) {
-  if (!h) return hlb_fail(HLB_ERR_ARG, "null solver");
-  const int64_t nb = hlb_reduce_partials(h->n);
-  double* out = h->d_red + nb + (h->n_iolets + 1);
-  CUDA_TRY(hlb_launch_reduce(h, h->f[h->cur], h->phase, h->t - 1, h->stepped, out, h->stream));
-  std::vector<double> host(1 + h->n_iolets);
+// Mass, fluxes and (monitor) per-iolet max |u| and mean rho of the current
+// state; one synchronisation.
+static int sums_impl(hlb_solver* h, double* mass, double* flux, bool monitor, double* u_max, double* rho_mean) {
+  const int K = h->n_iolets;
+  double* out = h->d_red + hlb_reduce_partials(h->n) + (K + 1);
+  CUDA_TRY(hlb_launch_reduce(h, h->f[h->cur], h->phase, h->t - 1, h->stepped, monitor, out, h->stream));
+  std::vector<double> host(1 + (size_t)K), mon(2 * (size_t)K);
   CUDA_TRY(cudaMemcpyAsync(host.data(), out, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, h->stream));
+  if (monitor)
+    CUDA_TRY(cudaMemcpyAsync(mon.data(), h->d_mon, sizeof(double) * mon.size(), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
   if (mass) *mass = host[0];
-  if (flux)
-    for (int k = 0; k < h->n_iolets; ++k) flux[k] = host[1 + k];
+  for (int k = 0; k < K; ++k) {
+    if (flux) flux[k] = host[(size_t)(1 + k)];
+    if (u_max) u_max[k] = mon[(size_t)k];
+    if (rho_mean) rho_mean[k] = mon[(size_t)(K + k)];
+  }
   if (!std::isfinite(host[0])) return hlb_fail(HLB_ERR_DIVERGED, "mass is not finite");
   return HLB_OK;
 }
 
 extern "C" int hlb_reduce(hlb_solver* h, double* mass, double* flux) {
-  return hlb_no_throw([&] { return hlb_reduce_impl(h, mass, flux); });
+  if (!h) return hlb_fail(HLB_ERR_ARG, "null solver");
+  return hlb_no_throw([&] { return sums_impl(h, mass, flux, false, nullptr, nullptr); });
 }
 
 static int hlb_iolet_monitor_impl(hlb_solver* h, double* flux, double* u_max, double* rho_mean) {
   if (!h) return hlb_fail(HLB_ERR_ARG, "null solver");
-  const int K = h->n_iolets;
-  if (K == 0) return HLB_OK;
-  if (flux) {
-    std::vector<double> fl((size_t)K);
-    int rc = hlb_reduce(h, nullptr, fl.data());
-    if (rc) return rc;
-    for (int k = 0; k < K; ++k) flux[k] = fl[(size_t)k];
+  if (h->n_iolets == 0 || (!flux && !u_max && !rho_mean)) return HLB_OK;
+  const size_t K = (size_t)h->n_iolets;
+  std::vector<double> f(K), u(K), r(K);
+  const int rc = sums_impl(h, nullptr, f.data(), true, u.data(), r.data());
+  if (rc == HLB_ERR_DIVERGED && !flux) {
+    // only the flux's caller is told of a run that has blown up
+  } else if (rc) {
+    return rc;
   }
-  if (!u_max && !rho_mean) return HLB_OK;
-  CUDA_TRY(hlb_launch_monitor(h, h->f[h->cur], h->phase, h->t - 1, h->d_mon, h->stream));
-  std::vector<double> host(2 * (size_t)K);
-  CUDA_TRY(cudaMemcpyAsync(host.data(), h->d_mon, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(cudaStreamSynchronize(h->stream));
-  for (int k = 0; k < K; ++k) {
-    if (u_max) u_max[k] = host[(size_t)k];
-    if (rho_mean) rho_mean[k] = host[(size_t)(K + k)];
+  for (size_t k = 0; k < K; ++k) {
+    if (flux) flux[k] = f[k];
+    if (u_max) u_max[k] = u[k];
+    if (rho_mean) rho_mean[k] = r[k];
   }
   return HLB_OK;
 }

@@ -304,23 +304,7 @@ __device__ __forceinline__ void collide(R* h, R omega) {
 // rho_s, u_s are the moments of s'(t-1) at x: BGK conserves mass and
 // momentum, so they equal the pre-collision moments at time t-1 that the
 // paper's push formulation uses for these boundaries.
-// Returns whether the site has an iolet link.
 // ---------------------------------------------------------------------------
-template <typename S>
-__device__ __forceinline__ bool gather_site(const S* __restrict__ fin, const int32_t* __restrict__ src,
-                                            int64_t n, int64_t sn, int64_t x, typename Real<S>::type* h) {
-  h[0] = ldpop(fin + x);
-  bool any_iolet = false;
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    int32_t s = ldidx(src + (int64_t)(i - 1) * sn + x);
-    int64_t a = s >= 0 ? (int64_t)i * n + s : (int64_t)opp(i) * n + x;
-    h[i] = ldpop(fin + a);
-    any_iolet |= s <= -2;
-  }
-  return any_iolet;
-}
-
 // Boundary values of iolet links at site x (rare: only iolet sites).  On
 // entry h[i] of an iolet link already holds s'_ibar(x) (the gather selects
 // the own opposite slot for every non-fluid source).  All index codes and
@@ -447,22 +431,6 @@ __device__ __forceinline__ R lane_iolet_value(int i, const LinkRec& L, R out, R 
 // opposite slot, or, for a non-fluid source, by x itself into slot i.
 __device__ __forceinline__ int64_t aa_addr(int i, int32_t s, int64_t n, int64_t x) {
   return s >= 0 ? (int64_t)opp(i) * n + s : (int64_t)i * n + x;
-}
-
-template <typename S, int MODE>
-__device__ __forceinline__ void load_state(const S* __restrict__ fin, const int32_t* __restrict__ src,
-                                           const LinkRec* __restrict__ links, const double* __restrict__ amp,
-                                           const StepParams& p, int64_t x, typename Real<S>::type* h) {
-  if (MODE == 1) {
-    if (gather_site<S>(fin, src, p.n, p.sn, x, h)) iolet_fixup<S>(fin, src, links, amp, p, x, h);
-  } else if (MODE == 2) {
-    h[0] = ldpop(fin + x);
-#pragma unroll
-    for (int i = 1; i < Q; ++i) h[i] = ldpop(fin + aa_addr(i, src[(int64_t)(i - 1) * p.sn + x], p.n, x));
-  } else {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) h[i] = ldpop(fin + (int64_t)i * p.n + x);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -652,5 +620,65 @@ __device__ __forceinline__ bool load_offsets(const IndexTables& ix, uint32_t sn,
     off[i] = fluid ? slot<WIDE>(i, n, s) : slot<WIDE>(opp(i), n, x);
   });
 }
+
+// f(t) at site x (tile `tile`), and the bits of the directions with a fluid
+// source (bit i - 1) when FLUID or the gather needs them.  The index rows are
+// addressed in 64 bits: these kernels read them once a call, not once a step.
+template <typename S, int MODE, bool CT, bool FLUID>
+__device__ __forceinline__ uint32_t load_state(const S* __restrict__ fin, const IndexTables& ix,
+                                               const LinkRec* __restrict__ links, const double* __restrict__ amp,
+                                               const StepParams& p, int64_t x, uint32_t tile, typename Real<S>::type* h) {
+  const int64_t n = p.n;
+  uint32_t fluid = 0;
+  h[0] = ldpop(fin + x);
+  bool iolet = false;
+  if (MODE != 0 || FLUID)
+    iolet = for_links<CT, true, LD_NC, MODE == 1>(ix, (uint32_t)p.sn, (uint32_t)x, tile, [&](int i, bool f, uint32_t s) {
+      if (FLUID) fluid |= f ? 1u << (i - 1) : 0u;
+      if (MODE == 1) h[i] = ldpop(fin + (f ? (int64_t)i * n + s : (int64_t)opp(i) * n + x));
+      if (MODE == 2) h[i] = ldpop(fin + (f ? (int64_t)opp(i) * n + s : (int64_t)i * n + x));
+    });
+  if (MODE == 0) {
+#pragma unroll
+    for (int i = 1; i < Q; ++i) h[i] = ldpop(fin + (int64_t)i * n + x);
+  }
+  if (MODE == 1 && iolet) iolet_fixup<S>(fin, ix.src, links, amp, p, x, h);
+  return fluid;
+}
+
+// ---------------------------------------------------------------------------
+// Sum of a site's 19 populations for the FP64 mass reductions.  GB300 runs
+// FP64 additions and conversions at 1/64 of the FP32 rate, and 38 of them a
+// site made the reduction take 2.8 times its memory time.  FP32 values are
+// therefore summed as an unevaluated pair hi + lo (Knuth's two-sum: the
+// rounding error of every addition is exact in FP32 and goes to lo), and the
+// pair is converted once.  lo is some 2^-24 of hi and carries a rounding error
+// of 2^-24 of itself, below what adding the site to a block's FP64 sum rounds
+// off.  A sum that leaves the FP32 range is taken again in FP64.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double site_sum(const double* h) {
+  double d = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) d += h[i];
+  return d;
+}
+__device__ __forceinline__ double site_sum(const float* h) {
+  float hi = h[0], lo = 0.f;
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const float s = __fadd_rn(hi, h[i]);
+    const float t = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(h[i], t)));
+    hi = s;
+  }
+  if (isfinite(hi)) return (double)hi + (double)lo;
+  double d = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) d += (double)h[i];
+  return d;
+}
+// Sites a thread of a mass reduction takes (a block: kMassSites x 256 sites),
+// so that the FP64 block sum is paid once for that many.
+constexpr int kMassSites = 4;
 
 }  // namespace hlb

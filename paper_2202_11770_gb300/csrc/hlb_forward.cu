@@ -25,7 +25,7 @@
 // GATHER_AA (AA buffer after an even step; boundaries already written).
 //
 // k_macros: the property cache of Section 3.2.2 step 7 (rho, u) plus WSS.
-// k_mass / k_flux / k_finish: FP64 reductions in a fixed order.
+// k_sums / k_sums_finish: FP64 mass, iolet fluxes and monitor in a fixed order.
 #include <math.h>
 
 #include "hlb_internal.h"
@@ -49,7 +49,10 @@ template <typename S> constexpr int pair_blocks() { return sizeof(S) == 4 ? 6 : 
 constexpr int kStepIoletLanes = 8;
 constexpr int kFixLanes = 16;
 
+constexpr int READ = 128;  // threads a block of the read-back kernels, one site each
+
 inline unsigned grid_for(int64_t n) { return (unsigned)((n + BLOCK - 1) / BLOCK); }
+inline int64_t mass_blocks(int64_t n) { return (n + kMassSites * BLOCK - 1) / (kMassSites * BLOCK); }
 
 // L2 prefetch hint: `bytes` (a multiple of 16) from a 16-byte aligned address.
 __device__ __forceinline__ void l2_prefetch(const void* q, uint32_t bytes) {
@@ -725,7 +728,7 @@ __global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_aa_odd2(S* A, const 
 // warps), the base, and each thread its offset; pairs of directions share a
 // word.  Padding entries (n <= x < sn) read as walls.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(CT_TILE) k_ctab_build(const int32_t* __restrict__ src, int64_t n, int64_t sn,
+__global__ void __launch_bounds__(CT_TILE, 3) k_ctab_build(const int32_t* __restrict__ src, int64_t n, int64_t sn,
                                                         uint32_t* __restrict__ ctab, int32_t* __restrict__ tbase,
                                                         uint32_t* __restrict__ rtab, int32_t* __restrict__ rbase,
                                                         int32_t* __restrict__ misfit) {
@@ -834,49 +837,64 @@ __global__ void __launch_bounds__(CT_TILE) k_ctab_build(const int32_t* __restric
 // ---------------------------------------------------------------------------
 // Read-back kernels.
 // ---------------------------------------------------------------------------
-// Density, velocity and wall shear stress of f(t).
-template <typename S, int MODE>
-__global__ void __launch_bounds__(BLOCK) k_macros(const S* __restrict__ fin, const int32_t* __restrict__ src,
-                                                  const LinkRec* __restrict__ links,
-                                                  const double* __restrict__ amp,
-                                                  const float* __restrict__ normal, const StepParams p,
-                                                  float* __restrict__ rho_out, float* __restrict__ u_out,
-                                                  float* __restrict__ wss_out) {
+// Density, velocity and wall shear stress of f(t).  Bound by DRAM: 76 bytes of
+// FP32 populations and 20 of output a site, and of the index the row form's
+// mask word tells wall links (4 bytes; the gathers 12) where the int32 table
+// took 72, twice in the gather modes.  20.0M sites, FP32, f(t) in place: 563 ->
+// 406 us; FP64, 200k sites: 189 -> 128 us (see the zero terms below).
+template <typename S, int MODE, bool CT>
+__global__ void __launch_bounds__(READ) k_macros(const S* __restrict__ fin, const IndexTables ix,
+                                                 const LinkRec* __restrict__ links, const double* __restrict__ amp,
+                                                 const float* __restrict__ normal, const StepParams p,
+                                                 float* __restrict__ rho_out, float* __restrict__ u_out,
+                                                 float* __restrict__ wss_out) {
   using R = typename Real<S>::type;
   const int64_t n = p.n;
-  const int64_t x = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
+  const int64_t x = (int64_t)blockIdx.x * READ + threadIdx.x;
   if (x >= n) return;
+  const uint32_t tile = (uint32_t)(x / CT_TILE);
   R h[Q];
-  load_state<S, MODE>(fin, src, links, amp, p, x, h);
+  uint32_t wall = 0;  // directions with a wall link
+  if (wss_out) {
+    wall = ~load_state<S, MODE, CT, true>(fin, ix, links, amp, p, x, tile, h) & ((1u << (Q - 1)) - 1u);
+    if (wall && ((__ldg(ix.imask + (x >> 5)) >> (x & 31)) & 1u)) {  // some of them iolet links
+#pragma unroll
+      for (int i = 1; i < Q; ++i)
+        if (((wall >> (i - 1)) & 1u) && ix.src[(int64_t)(i - 1) * p.sn + x] != -1) wall &= ~(1u << (i - 1));
+    }
+  } else {
+    load_state<S, MODE, CT, false>(fin, ix, links, amp, p, x, tile, h);
+  }
   Macro<R> m = moments<R>(h);
-  if (rho_out) rho_out[x] = (float)m.rho;
+  if (rho_out) __stcs(rho_out + x, (float)m.rho);
   if (u_out) {
-    u_out[x] = (float)m.ux;
-    u_out[n + x] = (float)m.uy;
-    u_out[2 * n + x] = (float)m.uz;
+    __stcs(u_out + x, (float)m.ux);
+    __stcs(u_out + n + x, (float)m.uy);
+    __stcs(u_out + 2 * n + x, (float)m.uz);
   }
   if (!wss_out) return;
-  // wall links and the fallback normal (sum of c_j over pull wall directions)
-  bool wall = false;
-  R nx = 0, ny = 0, nz = 0;
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    if (src[(int64_t)(i - 1) * p.sn + x] == -1) {
-      wall = true;
-      nx += R(cx(i));
-      ny += R(cy(i));
-      nz += R(cz(i));
-    }
-  }
   if (!wall) {
-    wss_out[x] = __int_as_float(0x7fc00000);  // NaN
+    __stcs(wss_out + x, __int_as_float(0x7fc00000));  // NaN
     return;
   }
+  R nx = 0, ny = 0, nz = 0;
   if (normal) {
     nx = R(normal[x]);
     ny = R(normal[n + x]);
     nz = R(normal[2 * n + x]);
   } else {
+    // fallback normal: the sum of c_j over the pull directions across a wall
+    int sx = 0, sy = 0, sz = 0;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const int b = (wall >> (i - 1)) & 1;
+      sx += cx(i) * b;
+      sy += cy(i) * b;
+      sz += cz(i) * b;
+    }
+    nx = R(sx);
+    ny = R(sy);
+    nz = R(sz);
     R l = sqrt(nx * nx + ny * ny + nz * nz);
     nx /= l; ny /= l; nz /= l;
   }
@@ -884,13 +902,15 @@ __global__ void __launch_bounds__(BLOCK) k_macros(const S* __restrict__ fin, con
   R pxx = 0, pyy = 0, pzz = 0, pxy = 0, pxz = 0, pyz = 0;
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
-    R d = h[i] - heq<R>(i, m.drho, m.rho, m.ux, m.uy, m.uz, usq15);
-    pxx += cx(i) * cx(i) * d;
-    pyy += cy(i) * cy(i) * d;
-    pzz += cz(i) * cz(i) * d;
-    pxy += cx(i) * cy(i) * d;
-    pxz += cx(i) * cz(i) * d;
-    pyz += cy(i) * cz(i) * d;
+    // only the components that c_i has: a product with 0 is not optimised
+    // away, and in FP64 the zero terms were half of the kernel's arithmetic
+    const R d = h[i] - heq<R>(i, m.drho, m.rho, m.ux, m.uy, m.uz, usq15);
+    if (cx(i)) pxx += d;
+    if (cy(i)) pyy += d;
+    if (cz(i)) pzz += d;
+    if (cx(i) && cy(i)) pxy = cx(i) * cy(i) > 0 ? pxy + d : pxy - d;
+    if (cx(i) && cz(i)) pxz = cx(i) * cz(i) > 0 ? pxz + d : pxz - d;
+    if (cy(i) && cz(i)) pyz = cy(i) * cz(i) > 0 ? pyz + d : pyz - d;
   }
   R k = -(R(1) - R(0.5) * omega_of<R>(p));
   R tx = k * (pxx * nx + pxy * ny + pxz * nz);
@@ -900,21 +920,26 @@ __global__ void __launch_bounds__(BLOCK) k_macros(const S* __restrict__ fin, con
   tx -= tn * nx;
   ty -= tn * ny;
   tz -= tn * nz;
-  wss_out[x] = (float)sqrt(tx * tx + ty * ty + tz * tz);
+  __stcs(wss_out + x, (float)sqrt(tx * tx + ty * ty + tz * tz));
 }
 
 // Shifted pre-collision state f(t) - w into out [19][n] (row < 0), or only
 // direction `row` into out [n].
-template <typename S, int MODE>
-__global__ void __launch_bounds__(BLOCK) k_state(const S* __restrict__ fin, const int32_t* __restrict__ src,
-                                                 const LinkRec* __restrict__ links,
-                                                 const double* __restrict__ amp, const StepParams p,
-                                                 S* __restrict__ out, int row) {
+template <typename S, int MODE, bool CT>
+__global__ void __launch_bounds__(READ) k_state(const S* __restrict__ fin, const IndexTables ix,
+                                                const LinkRec* __restrict__ links, const double* __restrict__ amp,
+                                                const StepParams p, S* __restrict__ out, int row) {
   using R = typename Real<S>::type;
-  const int64_t x = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
-  if (x >= p.n) return;
+  const int64_t n = p.n;
+  const int64_t x = (int64_t)blockIdx.x * READ + threadIdx.x;
+  if (x >= n) return;
+  if (MODE == 2 && row >= 0) {  // one direction of the AA gather: its own slot only
+    const int32_t s = row ? ix.src[(int64_t)(row - 1) * p.sn + x] : -1;
+    out[x] = fin[s >= 0 ? (int64_t)lane_opp(row) * n + s : (int64_t)row * n + x];
+    return;
+  }
   R h[Q];
-  load_state<S, MODE>(fin, src, links, amp, p, x, h);
+  load_state<S, MODE, CT, false>(fin, ix, links, amp, p, x, (uint32_t)(x / CT_TILE), h);
   if (row >= 0) {
 #pragma unroll
     for (int i = 0; i < Q; ++i)
@@ -922,7 +947,7 @@ __global__ void __launch_bounds__(BLOCK) k_state(const S* __restrict__ fin, cons
     return;
   }
 #pragma unroll
-  for (int i = 0; i < Q; ++i) out[(int64_t)i * p.n + x] = from_real<S>(h[i]);
+  for (int i = 0; i < Q; ++i) stpop<S>(out + (int64_t)i * n + x, h[i]);
 }
 
 // f = f^eq(rho0, u0) (Section 3.1 step 1), stored shifted.
@@ -960,39 +985,44 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return r;  // valid in thread 0
 }
 
-// Per-block sums of drho (mass - sites) over the sites [lo, hi) into
-// part[blockIdx.x].
-template <typename S, int MODE>
-__global__ void __launch_bounds__(BLOCK) k_mass(const S* __restrict__ fin, const int32_t* __restrict__ src,
-                                                const LinkRec* __restrict__ links,
-                                                const double* __restrict__ amp, const StepParams p, int64_t lo,
-                                                int64_t hi, double* __restrict__ part) {
+// The sums of a state in two launches.  k_sums: blocks [0, nmass) write the
+// sums of drho (mass - sites) over kMassSites x 256 sites of [lo, hi) each into
+// part[block]; in the A-B scheme the blocks after them take 256 link records
+// each and write the mass that each link lets in, recomputed from the
+// post-collision state s'(t-1), into lflux (the AA steps record it there
+// themselves).  With MON the last blocks take 256 entries of the iolets' site
+// lists each and write |u|^2 and rho of f(t) into msite.  k_sums_finish adds
+// them up in a fixed order.  One thread a link or site, whatever the number
+// of iolets: one block an iolet walked thousands of links in a chain of
+// dependent loads (26 us for 2 iolets of 2,000 links; now a few).
+template <typename S, int MODE, bool CT, bool MON>
+__global__ void __launch_bounds__(BLOCK) k_sums(const S* __restrict__ fin, const IndexTables ix,
+                                                const LinkRec* __restrict__ links, const double* __restrict__ amp,
+                                                const StepParams p, int64_t lo, int64_t hi, unsigned nmass,
+                                                unsigned nflux, int64_t nlinks, int64_t nlist,
+                                                const int32_t* __restrict__ ilist, double* __restrict__ part,
+                                                double* __restrict__ lflux, double* __restrict__ msite) {
   using R = typename Real<S>::type;
-  __shared__ double sh[BLOCK / 32];
-  const int64_t x = lo + (int64_t)blockIdx.x * BLOCK + threadIdx.x;
-  double d = 0;
-  if (x < hi) {
-    R h[Q];
-    load_state<S, MODE>(fin, src, links, amp, p, x, h);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) d += (double)h[i];
-  }
-  double s = block_sum(d, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// Per-iolet flux of the A-B scheme: one block per iolet over its link
-// records, in order, recomputed from the post-collision state s'(t-1).
-template <typename S>
-__global__ void __launch_bounds__(BLOCK) k_flux(const S* __restrict__ fin, const LinkRec* __restrict__ links,
-                                                const double* __restrict__ amp, const StepParams p,
-                                                const int64_t* __restrict__ begin, double* __restrict__ out) {
-  using R = typename Real<S>::type;
-  __shared__ double sh[BLOCK / 32];
-  const int k = blockIdx.x;
   const int64_t n = p.n;
-  double acc = 0;
-  for (int64_t r = begin[k] + threadIdx.x; r < begin[k + 1]; r += BLOCK) {
+  if (blockIdx.x < nmass) {
+    __shared__ double sh[BLOCK / 32];
+    double d = 0;
+    const int64_t x0 = lo + (int64_t)blockIdx.x * (kMassSites * BLOCK) + threadIdx.x;
+#pragma unroll 1
+    for (int k = 0; k < kMassSites; ++k) {
+      const int64_t x = x0 + k * BLOCK;
+      if (x >= hi) break;
+      R h[Q];
+      load_state<S, MODE, CT, false>(fin, ix, links, amp, p, x, (uint32_t)(x / CT_TILE), h);
+      d += site_sum(h);
+    }
+    const double s = block_sum(d, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    return;
+  }
+  if (blockIdx.x < nmass + nflux) {
+    const int64_t r = (int64_t)(blockIdx.x - nmass) * BLOCK + threadIdx.x;
+    if (r >= nlinks) return;
     const LinkRec L = links[r];
     const int64_t x = L.site;
     R own[Q];
@@ -1008,44 +1038,61 @@ __global__ void __launch_bounds__(BLOCK) k_flux(const S* __restrict__ fin, const
 #pragma unroll
     for (int i = 1; i < Q; ++i)
       if (i == j) val = iolet_value<R>(i, L, out, ms.rho, ms.ux, ms.uy, ms.uz, amp, p);
-    acc += (double)val - (double)out;
+    lflux[r] = (double)val - (double)out;
+    return;
   }
-  double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) out[1 + k] = s;
+  if (MON) {
+    const int64_t q = (int64_t)(blockIdx.x - nmass - nflux) * BLOCK + threadIdx.x;
+    if (q >= nlist) return;
+    const int64_t x = ilist[q];
+    R h[Q];
+    load_state<S, MODE, false, false>(fin, ix, links, amp, p, x, 0u, h);
+    const Macro<R> m = moments<R>(h);
+    msite[2 * q] = (double)m.ux * m.ux + (double)m.uy * m.uy + (double)m.uz * m.uz;
+    msite[2 * q + 1] = (double)m.rho;
+  }
 }
 
-// Per-iolet flux of the AA scheme: sum of the per-link values the last step
-// recorded, one block per iolet, in order.
-__global__ void __launch_bounds__(BLOCK) k_flux_sum(const double* __restrict__ lflux,
-                                                    const int64_t* __restrict__ begin, double* __restrict__ out) {
-  __shared__ double sh[BLOCK / 32];
-  const int k = blockIdx.x;
-  double acc = 0;
-  for (int64_t r = begin[k] + threadIdx.x; r < begin[k + 1]; r += BLOCK) acc += lflux[r];
-  double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) out[1 + k] = s;
-}
-
-// out[0] = n + sum of the per-block partials (fixed order).
-__global__ void __launch_bounds__(1024) k_finish(const double* __restrict__ part, int64_t nb, int64_t n,
-                                                 double* __restrict__ out) {
-  __shared__ double sh[32];
-  double v = 0;
-  for (int64_t b = threadIdx.x; b < nb; b += blockDim.x) v += part[b];
+// Final sums, a block each, in a fixed order: block 0, out[0] = n + the mass
+// partials; blocks 1 .. K, out[1 + k] = flux of iolet k, the sum over its link
+// records (0 when the state did not come from a step); then, for the monitor,
+// mon[k] = max |u| and mon[K + k] = mean rho over the sites linked to iolet k.
+__global__ void __launch_bounds__(512) k_sums_finish(const double* __restrict__ part, int64_t nb, int64_t n, int K,
+                                                     const double* __restrict__ lflux,
+                                                     const int64_t* __restrict__ begin, int have_flux,
+                                                     const double* __restrict__ msite,
+                                                     const int64_t* __restrict__ ioff, double* __restrict__ out,
+                                                     double* __restrict__ mon) {
+  __shared__ double sh[512 / 32];
+  const int b = blockIdx.x;
+  if (b <= K) {
+    const double* v = b == 0 ? part : lflux;
+    const int64_t lo = b == 0 ? 0 : begin[b - 1], hi = b == 0 ? nb : (have_flux ? begin[b] : begin[b - 1]);
+    double acc = 0;
+#pragma unroll 4
+    for (int64_t r = lo + threadIdx.x; r < hi; r += 512) acc += v[r];
+    const double s = block_sum(acc, sh);
+    if (threadIdx.x == 0) out[b] = b == 0 ? (double)n + s : s;
+    return;
+  }
+  const int k = b - K - 1;
+  const int64_t lo = ioff[k], hi = ioff[k + 1];
+  double umax = 0, rsum = 0;
+#pragma unroll 4
+  for (int64_t q = lo + threadIdx.x; q < hi; q += 512) {
+    umax = fmax(umax, sqrt(msite[2 * q]));
+    rsum += msite[2 * q + 1];
+  }
+  const double rs = block_sum(rsum, sh);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  for (int o = 16; o > 0; o >>= 1) umax = fmax(umax, __shfl_down_sync(FULL_MASK, umax, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = umax;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double r = 0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r += sh[k];
-    out[0] = (double)n + r;
+    for (int w = 1; w < 512 / 32; ++w) umax = fmax(umax, sh[w]);
+    mon[k] = umax;
+    mon[K + k] = hi > lo ? rs / (double)(hi - lo) : 0.0;
   }
-}
-
-__global__ void k_zero(double* p, int64_t m) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) p[i] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -1168,51 +1215,12 @@ struct MacroOp {
                          float* wss, cudaStream_t s) {
     StepParams p = h->params(tb);
     const float* nrm = h->has_normals ? h->d_normal : nullptr;
-    HLB_MODE_SWITCH(mode, (k_macros<S, M><<<grid_for(h->n), BLOCK, 0, s>>>((const S*)fin, h->d_src, h->d_links,
-                                                                             h->d_amp, nrm, p, rho, u, wss)));
+    const unsigned g = (unsigned)((h->n + READ - 1) / READ);
+    HLB_MODE_SWITCH(mode, ((h->compact ? k_macros<S, M, true> : k_macros<S, M, false>)<<<g, READ, 0, s>>>(
+                              (const S*)fin, h->index(), h->d_links, h->d_amp, nrm, p, rho, u, wss)));
     return cudaGetLastError();
   }
 };
-
-// Per-iolet monitor of f(t): block k walks the sites with a link to iolet k
-// (ilist[ioff[k] .. ioff[k+1])) and writes out[k] = max |u| and
-// out[K + k] = mean rho over them.  Per-thread partial sums run in a fixed
-// stride order and the block combines them in a fixed tree, so the result
-// does not depend on scheduling.
-template <typename S, int MODE>
-__global__ void __launch_bounds__(256) k_iolet_monitor(const S* __restrict__ fin, const int32_t* __restrict__ src,
-                                                       const LinkRec* __restrict__ links,
-                                                       const double* __restrict__ amp, const StepParams p,
-                                                       const int64_t* __restrict__ ioff,
-                                                       const int32_t* __restrict__ ilist, double* __restrict__ out) {
-  using R = typename Real<S>::type;
-  __shared__ double smax[256], ssum[256];
-  const int k = blockIdx.x;
-  const int64_t b = ioff[k], e = ioff[k + 1];
-  double umax = 0.0, rsum = 0.0;
-  for (int64_t q = b + threadIdx.x; q < e; q += blockDim.x) {
-    R h[Q];
-    load_state<S, MODE>(fin, src, links, amp, p, ilist[q], h);
-    const Macro<R> m = moments<R>(h);
-    const double u2 = (double)m.ux * m.ux + (double)m.uy * m.uy + (double)m.uz * m.uz;
-    umax = fmax(umax, sqrt(u2));
-    rsum += (double)m.rho;
-  }
-  smax[threadIdx.x] = umax;
-  ssum[threadIdx.x] = rsum;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + w]);
-      ssum[threadIdx.x] += ssum[threadIdx.x + w];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    out[k] = smax[0];
-    out[gridDim.x + k] = e > b ? ssum[0] / (double)(e - b) : 0.0;
-  }
-}
 
 // Windkessel outlets after a step (block k = iolet k; other iolets return).
 // q = -(mass that enters through outlet k to produce the current state f):
@@ -1297,8 +1305,7 @@ template <typename S>
 struct WkOp {
   static cudaError_t run(const hlb_solver* h, const void* fin, int64_t tb, bool shift, cudaStream_t s) {
     StepParams p = h->params(tb);
-    const int64_t nb = grid_for(h->n);
-    const int64_t* begin = (const int64_t*)(h->d_red + nb);  // link ranges stored after the reduction partials
+    const int64_t* begin = (const int64_t*)(h->d_red + hlb_reduce_partials(h->n));  // link ranges stored after the partials
     if (h->scheme == HLB_AA)
       return launch_pdl(k_wk_update<S, true>, (unsigned)h->n_iolets, BLOCK, s, (const S*)nullptr, h->d_links,
                         h->d_amp, p, begin, h->d_lflux, h->d_wkpar, h->d_wkstate, h->d_ioval, h->d_iovnext, 0);
@@ -1309,23 +1316,13 @@ struct WkOp {
 };
 
 template <typename S>
-struct MonitorOp {
-  static cudaError_t run(const hlb_solver* h, const void* fin, int mode, int64_t tb, double* out, cudaStream_t s) {
-    if (h->n_iolets == 0) return cudaSuccess;
-    StepParams p = h->params(tb);
-    HLB_MODE_SWITCH(mode, (k_iolet_monitor<S, M><<<h->n_iolets, 256, 0, s>>>(
-                              (const S*)fin, h->d_src, h->d_links, h->d_amp, p, h->d_ioff, h->d_ilist, out)));
-    return cudaGetLastError();
-  }
-};
-
-template <typename S>
 struct StateOp {
   static cudaError_t run(const hlb_solver* h, const void* fin, int mode, int64_t tb, void* out, int row,
                          cudaStream_t s) {
     StepParams p = h->params(tb);
-    HLB_MODE_SWITCH(mode, (k_state<S, M><<<grid_for(h->n), BLOCK, 0, s>>>((const S*)fin, h->d_src, h->d_links,
-                                                                            h->d_amp, p, (S*)out, row)));
+    const unsigned g = (unsigned)((h->n + READ - 1) / READ);
+    HLB_MODE_SWITCH(mode, ((h->compact ? k_state<S, M, true> : k_state<S, M, false>)<<<g, READ, 0, s>>>(
+                              (const S*)fin, h->index(), h->d_links, h->d_amp, p, (S*)out, row)));
     return cudaGetLastError();
   }
 };
@@ -1338,37 +1335,41 @@ struct InitOp {
   }
 };
 
+template <typename S, int MODE, bool CT>
+void launch_sums(const hlb_solver* h, const S* fin, const StepParams& p, bool links, bool monitor, cudaStream_t s) {
+  const int64_t lo = h->owned_lo, hi = h->owned_hi;
+  const unsigned nmass = (unsigned)mass_blocks(hi - lo), nflux = links ? grid_for(h->n_links) : 0u;
+  const unsigned nmon = monitor ? grid_for(h->n_ilist) : 0u;
+  (monitor ? k_sums<S, MODE, CT, true> : k_sums<S, MODE, CT, false>)<<<nmass + nflux + nmon, BLOCK, 0, s>>>(
+      fin, h->index(), h->d_links, h->d_amp, p, lo, hi, nmass, nflux, h->n_links, h->n_ilist, h->d_ilist, h->d_red,
+      h->d_lflux, h->d_msite);
+}
+
 template <typename S>
 struct ReduceOp {
-  static cudaError_t run(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux, double* out,
-                         cudaStream_t s) {
+  static cudaError_t run(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux, bool monitor,
+                         double* out, cudaStream_t s) {
     StepParams p = h->params(tb);
-    const int64_t nb = grid_for(h->n);
-    const int64_t lo = h->owned_lo, hi = h->owned_hi, nbo = grid_for(hi - lo);
-    double* part = h->d_red;
-    HLB_MODE_SWITCH(mode, (k_mass<S, M><<<(unsigned)nbo, BLOCK, 0, s>>>((const S*)fin, h->d_src, h->d_links,
-                                                                          h->d_amp, p, lo, hi, part)));
-    k_finish<<<1, 1024, 0, s>>>(part, nbo, hi - lo, out);
-    if (h->n_iolets > 0) {
-      const int64_t* begin = (const int64_t*)(h->d_red + nb);  // link ranges stored after the partials
-      if (!have_flux)
-        k_zero<<<1, 256, 0, s>>>(out + 1, h->n_iolets);
-      else if (h->scheme == HLB_AA)
-        k_flux_sum<<<(unsigned)h->n_iolets, BLOCK, 0, s>>>(h->d_lflux, begin, out);
-      else
-        k_flux<S><<<(unsigned)h->n_iolets, BLOCK, 0, s>>>((const S*)fin, h->d_links, h->d_amp, p, begin, out);
-    }
+    const int64_t owned = h->owned_hi - h->owned_lo;
+    // the A-B scheme's fluxes are recomputed; the AA steps have recorded them
+    const bool links = have_flux && h->scheme != HLB_AA && h->n_links > 0;
+    HLB_MODE_SWITCH(mode, (h->compact ? launch_sums<S, M, true>(h, (const S*)fin, p, links, monitor, s)
+                                      : launch_sums<S, M, false>(h, (const S*)fin, p, links, monitor, s)));
+    const int K = h->n_iolets;
+    const int64_t* begin = (const int64_t*)(h->d_red + hlb_reduce_partials(h->n));  // link ranges stored after the partials
+    k_sums_finish<<<(unsigned)(monitor ? 1 + 2 * K : 1 + K), 512, 0, s>>>(
+        h->d_red, mass_blocks(owned), owned, K, h->d_lflux, begin, have_flux ? 1 : 0, h->d_msite, h->d_ioff, out, h->d_mon);
     return cudaGetLastError();
   }
 };
 
 }  // namespace
 
-int64_t hlb_reduce_partials(int64_t n) { return (int64_t)grid_for(n); }
+int64_t hlb_reduce_partials(int64_t n) { return mass_blocks(n); }
 
 int64_t hlb_reduce_slots(int64_t n, int32_t n_iolets) {
   // per-block partials, iolet link ranges (int64, n_iolets + 1), final outputs (1 + n_iolets)
-  return (int64_t)grid_for(n) + (n_iolets + 1) + (1 + n_iolets);
+  return mass_blocks(n) + (n_iolets + 1) + (1 + n_iolets);
 }
 
 cudaError_t hlb_launch_step(const hlb_solver* h, const void* fin, void* fout, bool gather, int64_t tb,
@@ -1395,10 +1396,6 @@ cudaError_t hlb_launch_wk_reset(const hlb_solver* h, cudaStream_t s) {
                                                                    h->d_ioval, h->d_iovnext);
   return cudaGetLastError();
 }
-cudaError_t hlb_launch_monitor(const hlb_solver* h, const void* fin, int mode, int64_t tb, double* out,
-                               cudaStream_t s) {
-  return dispatch<MonitorOp>(h->precision, h, fin, mode, tb, out, s);
-}
 cudaError_t hlb_launch_state(const hlb_solver* h, const void* fin, int mode, int64_t tb, void* out, int row,
                              cudaStream_t s) {
   return dispatch<StateOp>(h->precision, h, fin, mode, tb, out, row, s);
@@ -1412,7 +1409,7 @@ cudaError_t hlb_launch_ctab(const hlb_solver* h, int32_t* misfit, cudaStream_t s
 cudaError_t hlb_launch_init(const hlb_solver* h, void* f, double rho0, const float* u0, cudaStream_t s) {
   return dispatch<InitOp>(h->precision, h, f, rho0, u0, s);
 }
-cudaError_t hlb_launch_reduce(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux,
+cudaError_t hlb_launch_reduce(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux, bool monitor,
                               double* out_dev, cudaStream_t s) {
-  return dispatch<ReduceOp>(h->precision, h, fin, mode, tb, have_flux, out_dev, s);
+  return dispatch<ReduceOp>(h->precision, h, fin, mode, tb, have_flux, monitor, out_dev, s);
 }

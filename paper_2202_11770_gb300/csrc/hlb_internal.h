@@ -79,6 +79,7 @@ struct hlb_solver {
   uint32_t* d_imask = nullptr;        // [(n + 31) / 32] bit x % 32 of word x / 32: site x has an iolet link
   int64_t* d_ioff = nullptr;          // [n_iolets + 1] ranges of d_ilist per iolet
   int32_t* d_ilist = nullptr;         // sites with a link to iolet k, ascending, iolet by iolet
+  double* d_msite = nullptr;          // [n_ilist][2] |u|^2 and rho of the sites of d_ilist (monitor scratch)
   double* d_mon = nullptr;            // [2][n_iolets] monitor outputs
   // Windkessel outlets: host flags, device parameters, model state and the
   // ghost densities the kernels read (io_val)
@@ -93,6 +94,7 @@ struct hlb_solver {
     return false;
   }
   int64_t n_iolet_sites = 0;
+  int64_t n_ilist = 0;                // entries of d_ilist
   int64_t red_slots = 0;
 
   hlb::IndexTables index() const { return {d_src, d_ctab, d_tbase, d_rtab, d_rbase, d_imask}; }
@@ -160,9 +162,6 @@ cudaError_t hlb_launch_wk_update(const hlb_solver* h, const void* fin, int64_t t
 // Windkessel outlets: forget the outflow history (q = 0) and reset the ghost
 // densities to the compliance state.
 cudaError_t hlb_launch_wk_reset(const hlb_solver* h, cudaStream_t s);
-// Per-iolet max |u| (out[k]) and mean rho (out[K + k]) over the sites linked to iolet k.
-cudaError_t hlb_launch_monitor(const hlb_solver* h, const void* fin, int mode, int64_t tb, double* out,
-                               cudaStream_t s);
 // Shifted pre-collision state into out [19][n] (row < 0) or direction `row` into out [n].
 cudaError_t hlb_launch_state(const hlb_solver* h, const void* fin, int mode, int64_t tb, void* out, int row,
                              cudaStream_t s);
@@ -177,8 +176,9 @@ cudaError_t hlb_launch_icode(const hlb_solver* h, cudaStream_t s);
 cudaError_t hlb_launch_ctab(const hlb_solver* h, int32_t* misfit, cudaStream_t s);
 // Equilibrium initialisation; u0 [3][n] device or null.
 cudaError_t hlb_launch_init(const hlb_solver* h, void* f, double rho0, const float* u0, cudaStream_t s);
-// Mass (out[0]) and per-iolet flux (out[1..]) in FP64.
-cudaError_t hlb_launch_reduce(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux,
+// Mass (out[0]) and per-iolet flux (out[1..]) in FP64; with `monitor` also
+// d_mon: per iolet max |u| (k) and mean rho (K + k) over the sites linked to it.
+cudaError_t hlb_launch_reduce(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux, bool monitor,
                               double* out_dev, cudaStream_t s);
 int64_t hlb_reduce_slots(int64_t n, int32_t n_iolets);
 // Number of per-block mass partials at the start of the reduction scratch.
