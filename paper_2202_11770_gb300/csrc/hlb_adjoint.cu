@@ -320,7 +320,7 @@ __device__ __forceinline__ typename Real<S>::type adjoint_iolet_site(const S* __
       if (code <= -2) {
         const LinkRec L = links[-code - 2];
         const R a = BC<R>::amp(p, amp, L.kind == 0 && L.group >= 0 ? L.group : 0);
-        h = lane_iolet_value<R>(i, L, h, rp, ux, uy, uz, a, p);
+        h = lane_iolet_value<R>(i, L, h, rp, ux, uy, uz, a, BC<R>::val(p, L.iolet), p);
       }
     } else if (dir) {
       h = ldpop(prev + (int64_t)i * n + x);

@@ -122,7 +122,7 @@ namespace {
 struct Layout {
   size_t f0 = 0, f1 = 0, src = 0, ctab = 0, tbase = 0, rtab = 0, rbase = 0, ctflag = 0, links = 0, amp = 0, ampf = 0, normal = 0, stage = 0, red = 0, lflux = 0, isites = 0, icode = 0, imask = 0, ioff = 0,
          ilist = 0, msite = 0, mon = 0, wkpar = 0, wkstate = 0,
-         ioval = 0, iovnext = 0, total = 0;
+         ioval = 0, iovnext = 0, word = 0, total = 0;
   int64_t n_links = 0;
   int32_t n_groups = 0;
 };
@@ -145,6 +145,7 @@ struct RowCheck {
   const char* msg = nullptr;
   std::vector<int64_t> per;
   std::vector<LinkRef> links;
+  bool mutual = true;  // x pulls from s in direction i, s from x in the opposite one (small lattices: checked)
 };
 
 void check_row(const hlb_lattice* L, int i, RowCheck* out) {
@@ -155,6 +156,7 @@ void check_row(const hlb_lattice* L, int i, RowCheck* out) {
     const int32_t s = row[x];
     if (s >= 0) {
       if (s >= n) { out->code = HLB_ERR_ARG; out->msg = "src index out of range"; return; }
+      if (n <= kMultiMaxSites) out->mutual &= L->src[(int64_t)(opp(i) - 1) * n + s] == x;
     } else if (s <= -2) {
       const int k = -s - 2;
       if (k >= L->n_iolets) { out->code = HLB_ERR_ARG; out->msg = "link code names a missing iolet"; return; }
@@ -169,7 +171,7 @@ void check_row(const hlb_lattice* L, int i, RowCheck* out) {
 }
 
 int validate(const hlb_lattice* L, const hlb_options* o, std::vector<int64_t>* per_iolet_links,
-             int64_t* n_iolet_sites, std::vector<LinkRef>* links_out = nullptr) {
+             int64_t* n_iolet_sites, std::vector<LinkRef>* links_out = nullptr, bool* mutual = nullptr) {
   if (!L || !o) return hlb_fail(HLB_ERR_ARG, "null lattice or options");
   if (L->n_sites < 1 || L->n_sites >= ((int64_t)1 << 31)) return hlb_fail(HLB_ERR_ARG, "n_sites must be in [1, 2^31)");
   if (!L->src || !L->xyz) return hlb_fail(HLB_ERR_ARG, "lattice needs xyz and src");
@@ -198,6 +200,8 @@ int validate(const hlb_lattice* L, const hlb_options* o, std::vector<int64_t>* p
   per_iolet_links->assign((size_t)std::max(1, (int)L->n_iolets), 0);
   for (const RowCheck& r : rows)
     if (r.code != HLB_OK) return hlb_fail(r.code, r.msg);
+  if (mutual)
+    for (const RowCheck& r : rows) *mutual &= r.mutual;
   std::vector<uint8_t> iolet_site((size_t)n, 0);
   *n_iolet_sites = 0;
   for (const RowCheck& r : rows) {
@@ -261,6 +265,9 @@ Layout layout(const hlb_lattice* L, const hlb_options* o, const std::vector<int6
   y.wkstate = off; off += align_up(sizeof(double) * 2 * (size_t)std::max(L->n_iolets, 1));
   y.ioval = off; off += align_up(sizeof(double) * (size_t)std::max(L->n_iolets, 1));
   y.iovnext = off; off += align_up(sizeof(double) * (size_t)std::max(L->n_iolets, 1));
+  if (n <= kMultiMaxSites && resolve_scheme(o->scheme, n) == HLB_PULL_AB) {
+    y.word = off; off += align_up(sizeof(uint64_t) * hlb_multi_words(n, y.n_links, L->n_iolets, o->precision));
+  }
   y.total = off;
   return y;
 }
@@ -320,7 +327,8 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   std::vector<int64_t> per;
   int64_t nis = 0;
   std::vector<LinkRef> links;
-  int rc = validate(L, o, &per, &nis, &links);
+  bool mutual = true;
+  int rc = validate(L, o, &per, &nis, &links, &mutual);
   if (rc) return rc;
   Layout y = layout(L, o, per, nis);
   if (!ws) return hlb_fail(HLB_ERR_WS, "null workspace");
@@ -397,6 +405,10 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   h->d_wkstate = (double*)(base + y.wkstate);
   h->d_ioval = (double*)(base + y.ioval);
   h->d_iovnext = (double*)(base + y.iovnext);
+  if (y.word && mutual) {
+    h->d_word = (uint64_t*)(base + y.word);
+    h->multi_blocks = hlb_multi_blocks(h);
+  }
   h->wk_on.assign((size_t)h->n_iolets, 0);
   h->n_iolet_sites = nis;
 
@@ -533,6 +545,8 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
     e = cudaMemcpyAsync(h->d_ioff, ioff.data(), sizeof(int64_t) * ioff.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !ilist.empty())
     e = cudaMemcpyAsync(h->d_ilist, ilist.data(), sizeof(int32_t) * ilist.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && h->multi_blocks > 0)
+    e = cudaMemsetAsync(h->d_word, 0, sizeof(uint64_t) * hlb_multi_words(n, y.n_links, h->n_iolets, h->precision), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_lflux, 0, sizeof(double) * (size_t)std::max<int64_t>(y.n_links, 1), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->f[0], 0, h->state_bytes(), st);  // rest: h = f - w = 0
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -682,6 +696,17 @@ extern "C" int hlb_step(hlb_solver* h, int64_t nsteps) {
   if (nsteps < 0) return hlb_fail(HLB_ERR_ARG, "negative step count");
   if (h->midstep) return hlb_fail(HLB_ERR_STATE, "a partial step (hlb_step_range) is not finished");
   for (int64_t s = 0; s < nsteps; ++s) {
+    if (h->scheme == HLB_PULL_AB && h->phase == HLB_READ_GATHER_AB) {
+      if (const int m = hlb_multi_steps(h, nsteps - s)) {
+        CUDA_TRY(hlb_launch_multi(h, h->f[h->cur], h->f[h->cur ^ 1], h->t, m, h->stream));
+        h->cur ^= 1;
+        h->t += m;
+        h->stepped = true;
+        if (h->any_wk()) CUDA_TRY(hlb_launch_wk_update(h, h->f[h->cur], h->t - 1, true, h->stream));
+        s += m - 1;
+        continue;
+      }
+    }
     if (h->scheme == HLB_AA) {
       // even step from f(t) in place, odd step from the swapped buffer
       const bool odd = h->phase == HLB_READ_GATHER_AA;

@@ -227,15 +227,31 @@ __device__ __forceinline__ R cdotu(int i, R ux, R uy, R uz) {
   return s;
 }
 
+__device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// Sums of products, whose two products the compiler may contract either way.
+// In FP64 its choice differed between kernels, so there the fused operations are
+// written out: every path gives the same bits.
+__device__ __forceinline__ float dot3(float ax, float ay, float az, float bx, float by, float bz) {
+  return ax * bx + ay * by + az * bz;
+}
+__device__ __forceinline__ double dot3(double ax, double ay, double az, double bx, double by, double bz) {
+  return fmadd(az, bz, fmadd(ay, by, ax * bx));
+}
+// 3 cu + 4.5 cu^2 - usq15 and the shifted equilibrium w (drho + rho b)
+__device__ __forceinline__ float heq_of(float w, float drho, float rho, float cu, float usq15) {
+  return w * (drho + rho * (3.f * cu + 4.5f * cu * cu - usq15));
+}
+__device__ __forceinline__ double heq_of(double w, double drho, double rho, double cu, double usq15) {
+  return w * fmadd(rho, fmadd(fmadd(4.5, cu, 3.0), cu, -usq15), drho);
+}
+
 // Shifted equilibrium of direction i at (drho, rho, u).
 template <typename R>
 __device__ __forceinline__ R heq(int i, R drho, R rho, R ux, R uy, R uz, R usq15) {
-  R cu = cdotu<R>(i, ux, uy, uz);
-  return wgt<R>(i) * (drho + rho * (R(3) * cu + R(4.5) * cu * cu - usq15));
+  return heq_of(wgt<R>(i), drho, rho, cdotu<R>(i, ux, uy, uz), usq15);
 }
-
-__device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // BGK collision (Eq. 3a, dt = 1): h'_i = h_i + omega (heq_i - h_i), handed to
 // emit(i, h'_i) direction by direction as each value is final.  Arranged by
@@ -344,13 +360,13 @@ __device__ __forceinline__ void iolet_fixup(const S* __restrict__ fin, const int
     } else {
       R gx = ux, gy = uy, gz = uz;
       if (!p.ghost_full_u) {
-        R un = gx * BC<R>::nx(iop) + gy * BC<R>::ny(iop) + gz * BC<R>::nz(iop);
+        R un = dot3(gx, gy, gz, BC<R>::nx(iop), BC<R>::ny(iop), BC<R>::nz(iop));
         gx = un * BC<R>::nx(iop);
         gy = un * BC<R>::ny(iop);
         gz = un * BC<R>::nz(iop);
       }
       R drho = BC<R>::val(p, L.iolet);
-      R usq15 = R(1.5) * (gx * gx + gy * gy + gz * gz);
+      R usq15 = R(1.5) * dot3(gx, gy, gz, gx, gy, gz);
       h[i] = heq<R>(i, drho, R(1) + drho, gx, gy, gz, usq15);
     }
   }
@@ -383,8 +399,7 @@ __device__ __forceinline__ R lane_cdotu(int i, R ux, R uy, R uz) {
 }
 template <typename R>
 __device__ __forceinline__ R lane_heq(int i, R drho, R rho, R ux, R uy, R uz, R usq15) {
-  R cu = lane_cdotu<R>(i, ux, uy, uz);
-  return lane_w<R>(i) * (drho + rho * (R(3) * cu + R(4.5) * cu * cu - usq15));
+  return heq_of(lane_w<R>(i), drho, rho, lane_cdotu<R>(i, ux, uy, uz), usq15);
 }
 // (sum v, sum v c) over lanes 0..18 in direction order; sgn = -1 sums -v c
 template <typename R>
@@ -401,24 +416,25 @@ __device__ __forceinline__ void lane_moment_sums(R v, R sgn, R* d, R* jx, R* jy,
   *d = a; *jx = x; *jy = y; *jz = z;
 }
 // Boundary value of the lane's iolet link (as iolet_fixup computes it):
-// `out` = s'_ibar(x); rho_s, u_s the moments of the stored post-collision state.
+// `out` = s'_ibar(x); rho_s, u_s the moments of the stored post-collision
+// state; val the iolet's boundary value (BC<R>::val).
 template <typename R>
-__device__ __forceinline__ R lane_iolet_value(int i, const LinkRec& L, R out, R rho_s, R ux, R uy, R uz, R a,
+__device__ __forceinline__ R lane_iolet_value(int i, const LinkRec& L, R out, R rho_s, R ux, R uy, R uz, R a, R val,
                                               const StepParams& p) {
   const IoletParam& iop = p.io[L.iolet];
   if (L.kind == 0) {
     R rho = p.ladd_rho_one ? R(1) : rho_s;
-    return out + BC<R>::coef(L) * rho * a * BC<R>::val(p, L.iolet);
+    return out + BC<R>::coef(L) * rho * a * val;
   }
   R gx = ux, gy = uy, gz = uz;
   if (!p.ghost_full_u) {
-    R un = gx * BC<R>::nx(iop) + gy * BC<R>::ny(iop) + gz * BC<R>::nz(iop);
+    R un = dot3(gx, gy, gz, BC<R>::nx(iop), BC<R>::ny(iop), BC<R>::nz(iop));
     gx = un * BC<R>::nx(iop);
     gy = un * BC<R>::ny(iop);
     gz = un * BC<R>::nz(iop);
   }
-  R drho = BC<R>::val(p, L.iolet);
-  R usq15 = R(1.5) * (gx * gx + gy * gy + gz * gz);
+  R drho = val;
+  R usq15 = R(1.5) * dot3(gx, gy, gz, gx, gy, gz);
   return lane_heq<R>(i, drho, R(1) + drho, gx, gy, gz, usq15);
 }
 
@@ -680,5 +696,25 @@ __device__ __forceinline__ double site_sum(const float* h) {
 // Sites a thread of a mass reduction takes (a block: kMassSites x 256 sites),
 // so that the FP64 block sum is paid once for that many.
 constexpr int kMassSites = 4;
+
+// Post-collision population of direction i from the site's sums, with the
+// operations of collide_emit.
+template <typename R>
+__device__ __forceinline__ R iolet_lane_out(int i, R h, R omega, R drho, R rho, R ux, R uy, R uz, R usq15) {
+  const R om1 = R(1) - omega;
+  if (i == 0) {
+    const R ow = omega * wgt<R>(0);
+    return fmadd(om1, h, fmadd(-(ow * rho), usq15, ow * drho));
+  }
+  const int ip = 2 * ((i - 1) >> 1) + 1;
+  const R ow = omega * (ip <= 6 ? wgt<R>(1) : wgt<R>(7));
+  const R cu = lane_cdotu<R>(ip, ux, uy, uz);
+  const R a = fmadd(R(4.5) * cu, cu, -usq15);
+  return fmadd(om1, h, fmadd(ow * rho, fmadd((i & 1) ? R(3) : R(-3), cu, a), ow * drho));
+}
+// Lanes a site for the iolet sites of the pull step: a site's 19 directions
+// spread over them, up to ceil(19 / lanes) a lane (measured on the 20M-site
+// tree: BF16 step 418 us at 32, 411 at 16, 405 at 8).
+constexpr int kStepIoletLanes = 8;
 
 }  // namespace hlb

@@ -42,11 +42,8 @@ constexpr int BLOCK = 256;
 constexpr int PAIR = CT_TILE / 2;
 template <typename S> constexpr int pair_blocks() { return sizeof(S) == 4 ? 6 : 7; }
 
-// Lanes a site for the iolet sites: a site's 19 directions spread over them,
-// up to ceil(19 / lanes) a lane.  Measured on the 20M-site tree: the pull
-// step's iolet sites 8 lanes (BF16 step 411 -> 405 us against 16, 418 at 32),
-// the AA iolet pass 16 (8 lanes 1-2 us slower a step, 32 lanes 3 us slower).
-constexpr int kStepIoletLanes = 8;
+// Lanes a site in the AA iolet pass (8 lanes 1-2 us slower a step on the
+// 20M-site tree, 32 lanes 3 us slower).
 constexpr int kFixLanes = 16;
 
 constexpr int READ = 128;  // threads a block of the read-back kernels, one site each
@@ -117,21 +114,6 @@ __global__ void __launch_bounds__(BLOCK) k_step_local(const S* __restrict__ fin,
   collide_emit<R>(h, omega_of<R>(p), [&](int i, R v) { stpop<S>(fout + (int64_t)i * n + x, v); });
 }
 
-// Post-collision population of direction i from the site's sums, with the
-// operations of collide_emit.
-template <typename R>
-__device__ __forceinline__ R iolet_lane_out(int i, R h, R omega, R drho, R rho, R ux, R uy, R uz, R usq15) {
-  const R om1 = R(1) - omega;
-  if (i == 0) {
-    const R ow = omega * wgt<R>(0);
-    return fmadd(om1, h, fmadd(-(ow * rho), usq15, ow * drho));
-  }
-  const int ip = 2 * ((i - 1) >> 1) + 1;
-  const R ow = omega * (ip <= 6 ? wgt<R>(1) : wgt<R>(7));
-  const R cu = lane_cdotu<R>(ip, ux, uy, uz);
-  const R a = fmadd(R(4.5) * cu, cu, -usq15);
-  return fmadd(om1, h, fmadd(ow * rho, fmadd((i & 1) ? R(3) : R(-3), cu, a), ow * drho));
-}
 // The same step for the sites with iolet links, kStepIoletLanes lanes a
 // site, lane h holding directions h, h + lanes, ... (gather, boundary value,
 // collision).  Moments and collision sums run over the directions in the
@@ -180,7 +162,7 @@ __device__ __forceinline__ void step_iolet_site(const S* __restrict__ fin, S* __
   const R ux = jx / rho_s, uy = jy / rho_s, uz = jz / rho_s;
 #pragma unroll
   for (int e = 0; e < NE; ++e)
-    if (c[e] <= -2) h[e] = lane_iolet_value<R>(e * W + hl, L[e], h[e], rho_s, ux, uy, uz, a[e], p);
+    if (c[e] <= -2) h[e] = lane_iolet_value<R>(e * W + hl, L[e], h[e], rho_s, ux, uy, uz, a[e], BC<R>::val(p, L[e].iolet), p);
   // collision: sums over opposite pairs as collide_emit forms them
   const R omega = omega_of<R>(p);
   R drho = __shfl_sync(FULL_MASK, h[0], 0, W), cjx = R(0), cjy = R(0), cjz = R(0);
@@ -527,13 +509,13 @@ __device__ __forceinline__ R iolet_value(int i, const LinkRec& L, R out, R rho, 
   }
   R gx = ux, gy = uy, gz = uz;
   if (!p.ghost_full_u) {
-    R un = gx * BC<R>::nx(io) + gy * BC<R>::ny(io) + gz * BC<R>::nz(io);
+    R un = dot3(gx, gy, gz, BC<R>::nx(io), BC<R>::ny(io), BC<R>::nz(io));
     gx = un * BC<R>::nx(io);
     gy = un * BC<R>::ny(io);
     gz = un * BC<R>::nz(io);
   }
   R drho = BC<R>::val(p, L.iolet);
-  R usq15 = R(1.5) * (gx * gx + gy * gy + gz * gz);
+  R usq15 = R(1.5) * dot3(gx, gy, gz, gx, gy, gz);
   return heq<R>(i, drho, R(1) + drho, gx, gy, gz, usq15);
 }
 
@@ -606,7 +588,7 @@ __global__ void __launch_bounds__(256, 8) k_aa_fix(S* A, const int32_t* __restri
   for (int e = 0; e < NE; ++e) {
     const int i = e * W + hl;
     if (c[e] <= -2) {
-      const R val = lane_iolet_value<R>(i, L[e], v[e], rho, ux, uy, uz, a[e], p);
+      const R val = lane_iolet_value<R>(i, L[e], v[e], rho, ux, uy, uz, a[e], BC<R>::val(p, L[e].iolet), p);
       lflux[-c[e] - 2] = (double)val - (double)v[e];
       A[(int64_t)i * n + x] = from_real<S>(val);
     }

@@ -88,6 +88,10 @@ struct hlb_solver {
   double* d_wkstate = nullptr;        // [n_iolets][2] rho_c, q (outflow of the last step)
   double* d_ioval = nullptr;          // [n_iolets] ghost density - 1 the kernels read (io_val)
   double* d_iovnext = nullptr;        // [n_iolets] pull A-B: the one after it (boundaries lag a step)
+  // many steps a launch (hlb_multi.cu), small lattices with mutual links only
+  uint64_t* d_word = nullptr;         // words that pass between sites (hlb_multi_words)
+  int multi_blocks = 0;               // blocks that fit on the device at once, 0: steps are launched one by one
+  uint32_t multi_tag = 1;             // number of the next such step (0: never written)
   bool any_wk() const {
     for (int v : wk_on)
       if (v) return true;
@@ -139,6 +143,20 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+
+// ---- many steps a launch (hlb_multi.cu) ----
+constexpr int kMultiVals = 2048;           // boundary values [step][iolet] of a launch
+constexpr int kMultiMin = 4;               // fewer steps are launched one by one
+constexpr int64_t kMultiSites = 24000;     // sites up to which it is the faster form (hlb_multi_steps)
+constexpr int64_t kMultiMaxSites = 100000; // sites of a lattice that may fit on the device at once
+// 64-bit words of device scratch.
+size_t hlb_multi_words(int64_t n, int64_t n_links, int32_t n_iolets, int32_t precision);
+// Blocks of the solver's kernel that the device holds at once (0: not available).
+int hlb_multi_blocks(const hlb_solver* h);
+// Steps that the next launch may take towards `left` more, 0: launch them one by one.
+int hlb_multi_steps(const hlb_solver* h, int64_t left);
+// m pull A-B gather steps from `in`, which holds s'(t - 1); the last is stored to `out`.
+cudaError_t hlb_launch_multi(hlb_solver* h, const void* in, void* out, int64_t t, int m, cudaStream_t s);
 
 // ---- launchers (hlb_forward.cu) ----
 // One pull A-B time step from fin into fout (gather: fin holds s'(t-1)).
