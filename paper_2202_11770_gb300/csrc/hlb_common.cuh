@@ -253,19 +253,83 @@ __device__ __forceinline__ R heq(int i, R drho, R rho, R ux, R uy, R uz, R usq15
   return heq_of(wgt<R>(i), drho, rho, cdotu<R>(i, ux, uy, uz), usq15);
 }
 
+// What the collision of a site takes from its sums drho = sum h and j = sum h c:
+// rest(h) is the post-collision population of direction 0, side(c, .., h) of a
+// direction of weight class c (1: axis, 2: diagonal) given its pair's c.u or c.j
+// and the sign that tells the pair's two directions apart.
+template <typename R> struct Bgk;
+
+// FP32.  A pair shares a = 4.5 (c.u)^2 - 1.5 u.u, and its two equilibria are
+// w (drho + rho (a +- 3 c.u)); h' = (1 - omega) h + omega heq, with omega w rho
+// and omega w drho formed once per weight class, is two fused multiply-adds
+// per direction.
+template <> struct Bgk<float> {
+  float ux, uy, uz, usq15, om1, wr[3], wd[3];  // wr, wd: omega w rho, omega w drho for w = 1/3, 1/18, 1/36
+  __device__ __forceinline__ Bgk(float drho, float jx, float jy, float jz, float omega) {
+    const float rho = 1.f + drho;
+    const float inv = 1.f / rho;
+    ux = jx * inv;
+    uy = jy * inv;
+    uz = jz * inv;
+    usq15 = 1.5f * fmadd(uz, uz, fmadd(uy, uy, ux * ux));
+    om1 = 1.f - omega;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float ow = omega * wgt<float>(c == 0 ? 0 : (c == 1 ? 1 : 7));
+      wr[c] = ow * rho;
+      wd[c] = ow * drho;
+    }
+  }
+  __device__ __forceinline__ float rest(float h) const { return fmadd(om1, h, fmadd(-wr[0], usq15, wd[0])); }
+  __device__ __forceinline__ float side(int c, float cu, float k, float h) const {
+    const float a = fmadd(4.5f * cu, cu, -usq15);
+    return fmadd(om1, h, fmadd(c == 1 ? wr[1] : wr[2], fmadd(k, cu, a), c == 1 ? wd[1] : wd[2]));
+  }
+};
+
+// FP64, which GB300 runs at 1/64 of the FP32 rate: the FP64 step kernels are
+// bound by the number of these operations.  With rho u = j a pair's two values
+// are (1 - omega) h + e +- b c.j, e = T (c.j)^2 + A, where A = w omega (drho -
+// 1.5 j.j / rho), T = 4.5 w omega / rho and b = 3 w omega per weight class: six
+// operations a pair after c.j, none of them for u.
+template <> struct Bgk<double> {
+  double jx, jy, jz, om1, A[3], T[2], B[2];  // T, B: w = 1/18, 1/36
+  __device__ __forceinline__ Bgk(double drho, double x, double y, double z, double omega) : jx(x), jy(y), jz(z) {
+    const double t = omega * (1.0 / (1.0 + drho));
+    const double jj = fmadd(jz, jz, fmadd(jy, jy, jx * jx));
+    const double a = fmadd(-1.5 * t, jj, omega * drho);
+    om1 = 1.0 - omega;
+    A[0] = a * (1.0 / 3.0);
+    A[1] = a * (1.0 / 18.0);
+    A[2] = 0.5 * A[1];
+    T[0] = 0.25 * t;
+    T[1] = 0.125 * t;
+    B[0] = omega * (1.0 / 6.0);
+    B[1] = 0.5 * B[0];
+  }
+  __device__ __forceinline__ double rest(double h) const { return fmadd(om1, h, A[0]); }
+  __device__ __forceinline__ double side(int c, double cj, double sign, double h) const {
+    const double e = fmadd((c == 1 ? T[0] : T[1]) * cj, cj, c == 1 ? A[1] : A[2]);
+    return fmadd(om1, h, fmadd(sign * (c == 1 ? B[0] : B[1]), cj, e));
+  }
+};
+
+// c.v of direction i, whose first nonzero component is positive (odd i).
+template <typename R>
+__device__ __forceinline__ R cdot_pair(int i, R vx, R vy, R vz) {
+  if (cx(i)) return cy(i) ? (cy(i) > 0 ? vx + vy : vx - vy) : (cz(i) ? (cz(i) > 0 ? vx + vz : vx - vz) : vx);
+  if (cy(i)) return cz(i) ? (cz(i) > 0 ? vy + vz : vy - vz) : vy;
+  return vz;
+}
+
 // BGK collision (Eq. 3a, dt = 1): h'_i = h_i + omega (heq_i - h_i), handed to
 // emit(i, h'_i) direction by direction as each value is final.  Arranged by
-// opposite pairs (2p+1, 2p+2), whose c.u differ in sign only:
-//  * pair sums and differences give drho = h_0 + sum (h_2p+1 + h_2p+2) and
-//    j = sum (h_2p+1 - h_2p+2) c_{2p+1};
-//  * a pair shares a = 4.5 (c.u)^2 - 1.5 u.u, and its two equilibria are
-//    w (drho + rho (a +- 3 c.u));
-//  * h' = (1 - omega) h + omega heq, with omega w rho and omega w drho formed
-//    once per weight class, is two fused multiply-adds per direction.
-// About 140 FP32 instructions a site against 210 for the direction-by-
-// direction form, in kernels whose 16-bit variants are issue-bound; emitting
-// each pair as soon as it is final lets a kernel store it and free its
-// registers.
+// opposite pairs (2p+1, 2p+2), whose c.u differ in sign only: pair sums and
+// differences give drho = h_0 + sum (h_2p+1 + h_2p+2) and j = sum (h_2p+1 -
+// h_2p+2) c_{2p+1}, and Bgk the rest.  About 140 FP32 instructions a site
+// against 210 for the direction-by-direction form, in kernels whose 16-bit
+// variants are issue-bound; emitting each pair as soon as it is final lets a
+// kernel store it and free its registers.
 template <typename R, typename Emit>
 __device__ __forceinline__ void collide_emit(const R* h, R omega, Emit&& emit) {
   R drho = h[0], jx = R(0), jy = R(0), jz = R(0);
@@ -278,26 +342,20 @@ __device__ __forceinline__ void collide_emit(const R* h, R omega, Emit&& emit) {
     if (cy(i)) jy = cy(i) > 0 ? jy + dp : jy - dp;
     if (cz(i)) jz = cz(i) > 0 ? jz + dp : jz - dp;
   }
-  const R rho = R(1) + drho;
-  const R inv = R(1) / rho;
-  const R ux = jx * inv, uy = jy * inv, uz = jz * inv;
-  const R usq15 = R(1.5) * fmadd(uz, uz, fmadd(uy, uy, ux * ux));
-  const R om1 = R(1) - omega;
-  R wr[3], wd[3];  // omega w rho, omega w drho for w = 1/3, 1/18, 1/36
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const R ow = omega * wgt<R>(c == 0 ? 0 : (c == 1 ? 1 : 7));
-    wr[c] = ow * rho;
-    wd[c] = ow * drho;
-  }
-  emit(0, fmadd(om1, h[0], fmadd(-wr[0], usq15, wd[0])));
+  const Bgk<R> b(drho, jx, jy, jz, omega);
+  emit(0, b.rest(h[0]));
 #pragma unroll
   for (int p = 0; p < 9; ++p) {
     const int i = 2 * p + 1, c = i <= 6 ? 1 : 2;
-    const R cu = cdotu<R>(i, ux, uy, uz);
-    const R a = fmadd(R(4.5) * cu, cu, -usq15);
-    emit(i, fmadd(om1, h[i], fmadd(wr[c], fmadd(R(3), cu, a), wd[c])));
-    emit(i + 1, fmadd(om1, h[i + 1], fmadd(wr[c], fmadd(R(-3), cu, a), wd[c])));
+    if constexpr (sizeof(R) == 4) {
+      const R cu = cdotu<R>(i, b.ux, b.uy, b.uz);
+      emit(i, b.side(c, cu, R(3), h[i]));
+      emit(i + 1, b.side(c, cu, R(-3), h[i + 1]));
+    } else {
+      const R cj = cdot_pair<R>(i, b.jx, b.jy, b.jz);
+      emit(i, b.side(c, cj, R(1), h[i]));
+      emit(i + 1, b.side(c, cj, R(-1), h[i + 1]));
+    }
   }
 }
 
@@ -697,20 +755,15 @@ __device__ __forceinline__ double site_sum(const float* h) {
 // so that the FP64 block sum is paid once for that many.
 constexpr int kMassSites = 4;
 
-// Post-collision population of direction i from the site's sums, with the
-// operations of collide_emit.
+// Post-collision population of a lane's direction i (collide_emit's operations).
 template <typename R>
-__device__ __forceinline__ R iolet_lane_out(int i, R h, R omega, R drho, R rho, R ux, R uy, R uz, R usq15) {
-  const R om1 = R(1) - omega;
-  if (i == 0) {
-    const R ow = omega * wgt<R>(0);
-    return fmadd(om1, h, fmadd(-(ow * rho), usq15, ow * drho));
-  }
-  const int ip = 2 * ((i - 1) >> 1) + 1;
-  const R ow = omega * (ip <= 6 ? wgt<R>(1) : wgt<R>(7));
-  const R cu = lane_cdotu<R>(ip, ux, uy, uz);
-  const R a = fmadd(R(4.5) * cu, cu, -usq15);
-  return fmadd(om1, h, fmadd(ow * rho, fmadd((i & 1) ? R(3) : R(-3), cu, a), ow * drho));
+__device__ __forceinline__ R iolet_lane_out(int i, R h, const Bgk<R>& b) {
+  if (i == 0) return b.rest(h);
+  const int ip = 2 * ((i - 1) >> 1) + 1, c = ip <= 6 ? 1 : 2;
+  if constexpr (sizeof(R) == 4)
+    return b.side(c, lane_cdotu<R>(ip, b.ux, b.uy, b.uz), (i & 1) ? R(3) : R(-3), h);
+  else
+    return b.side(c, lane_cdotu<R>(ip, b.jx, b.jy, b.jz), (i & 1) ? R(1) : R(-1), h);
 }
 // Lanes a site for the iolet sites of the pull step: a site's 19 directions
 // spread over them, up to ceil(19 / lanes) a lane (measured on the 20M-site

@@ -176,15 +176,12 @@ __device__ __forceinline__ void step_iolet_site(const S* __restrict__ fin, S* __
     if (cy(ip)) cjy = cy(ip) > 0 ? cjy + dp : cjy - dp;
     if (cz(ip)) cjz = cz(ip) > 0 ? cjz + dp : cjz - dp;
   }
-  const R rho = R(1) + drho;
-  const R inv = R(1) / rho;
-  const R cux = cjx * inv, cuy = cjy * inv, cuz = cjz * inv;
-  const R usq15 = R(1.5) * fmadd(cuz, cuz, fmadd(cuy, cuy, cux * cux));
+  const Bgk<R> bgk(drho, cjx, cjy, cjz, omega);
   if (!live) return;
 #pragma unroll
   for (int e = 0; e < NE; ++e) {
     const int i = e * W + hl;
-    if (i < Q) stpop<S>(fout + (int64_t)i * n + x, iolet_lane_out<R>(i, h[e], omega, drho, rho, cux, cuy, cuz, usq15));
+    if (i < Q) stpop<S>(fout + (int64_t)i * n + x, iolet_lane_out<R>(i, h[e], bgk));
   }
 }
 

@@ -241,15 +241,12 @@ __device__ __forceinline__ void iolet_block(const S* in, S* out, const MultiArgs
       if (cy(ip)) cjy = cy(ip) > 0 ? cjy + dp : cjy - dp;
       if (cz(ip)) cjz = cz(ip) > 0 ? cjz + dp : cjz - dp;
     }
-    const R rho = R(1) + drho;
-    const R inv = R(1) / rho;
-    const R cux = cjx * inv, cuy = cjy * inv, cuz = cjz * inv;
-    const R usq15 = R(1.5) * fmadd(cuz, cuz, fmadd(cuy, cuy, cux * cux));
+    const Bgk<R> bgk(drho, cjx, cjy, cjz, omega);
 #pragma unroll
     for (int e = 0; e < NE; ++e) {
       const int i = e * W + hl;
       if (i >= Q) continue;
-      own[e] = rounded<S>(iolet_lane_out<R>(i, h[e], omega, drho, rho, cux, cuy, cuz, usq15));
+      own[e] = rounded<S>(iolet_lane_out<R>(i, h[e], bgk));
       if (!live) continue;
       if (i > 0 && !last) WD::store(put + (uint64_t)((uint32_t)(i - 1) * n + x) * WD::N, own[e], tag);
       if (last) out[(uint32_t)i * n + x] = from_real<S>(own[e]);
