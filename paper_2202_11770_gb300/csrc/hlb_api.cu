@@ -121,7 +121,7 @@ namespace {
 
 struct Layout {
   size_t f0 = 0, f1 = 0, src = 0, ctab = 0, tbase = 0, rtab = 0, rbase = 0, ctflag = 0, links = 0, amp = 0, ampf = 0, normal = 0, stage = 0, red = 0, lflux = 0, isites = 0, icode = 0, imask = 0, ioff = 0,
-         ilist = 0, msite = 0, mon = 0, wkpar = 0, wkstate = 0,
+         ilist = 0, msite = 0, wkpar = 0, wkstate = 0,
          ioval = 0, iovnext = 0, word = 0, total = 0;
   int64_t n_links = 0;
   int32_t n_groups = 0;
@@ -260,7 +260,6 @@ Layout layout(const hlb_lattice* L, const hlb_options* o, const std::vector<int6
   y.ioff = off; off += align_up(sizeof(int64_t) * (size_t)(L->n_iolets + 1));
   y.ilist = off; off += align_up(sizeof(int32_t) * (size_t)std::max<int64_t>(y.n_links, 1));  // >= sites per iolet
   y.msite = off; off += align_up(sizeof(double) * 2 * (size_t)std::max<int64_t>(y.n_links, 1));
-  y.mon = off; off += align_up(sizeof(double) * 2 * (size_t)std::max(L->n_iolets, 1));
   y.wkpar = off; off += align_up(sizeof(double) * 4 * (size_t)std::max(L->n_iolets, 1));
   y.wkstate = off; off += align_up(sizeof(double) * 2 * (size_t)std::max(L->n_iolets, 1));
   y.ioval = off; off += align_up(sizeof(double) * (size_t)std::max(L->n_iolets, 1));
@@ -400,7 +399,6 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   h->d_ioff = (int64_t*)(base + y.ioff);
   h->d_ilist = (int32_t*)(base + y.ilist);
   h->d_msite = (double*)(base + y.msite);
-  h->d_mon = (double*)(base + y.mon);
   h->d_wkpar = (double*)(base + y.wkpar);
   h->d_wkstate = (double*)(base + y.wkstate);
   h->d_ioval = (double*)(base + y.ioval);
@@ -757,16 +755,14 @@ static int sums_impl(hlb_solver* h, double* mass, double* flux, bool monitor, do
   const int K = h->n_iolets;
   double* out = h->d_red + hlb_reduce_partials(h->n) + (K + 1);
   CUDA_TRY(hlb_launch_reduce(h, h->f[h->cur], h->phase, h->t - 1, h->stepped, monitor, out, h->stream));
-  std::vector<double> host(1 + (size_t)K), mon(2 * (size_t)K);
+  std::vector<double> host((size_t)(monitor ? 1 + 3 * K : 1 + K));
   CUDA_TRY(cudaMemcpyAsync(host.data(), out, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, h->stream));
-  if (monitor)
-    CUDA_TRY(cudaMemcpyAsync(mon.data(), h->d_mon, sizeof(double) * mon.size(), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
   if (mass) *mass = host[0];
   for (int k = 0; k < K; ++k) {
     if (flux) flux[k] = host[(size_t)(1 + k)];
-    if (u_max) u_max[k] = mon[(size_t)k];
-    if (rho_mean) rho_mean[k] = mon[(size_t)(K + k)];
+    if (u_max) u_max[k] = host[(size_t)(1 + K + k)];
+    if (rho_mean) rho_mean[k] = host[(size_t)(1 + 2 * K + k)];
   }
   if (!std::isfinite(host[0])) return hlb_fail(HLB_ERR_DIVERGED, "mass is not finite");
   return HLB_OK;

@@ -49,7 +49,7 @@ constexpr int kFixLanes = 16;
 constexpr int READ = 128;  // threads a block of the read-back kernels, one site each
 
 inline unsigned grid_for(int64_t n) { return (unsigned)((n + BLOCK - 1) / BLOCK); }
-inline int64_t mass_blocks(int64_t n) { return (n + kMassSites * BLOCK - 1) / (kMassSites * BLOCK); }
+inline int64_t mass_blocks(int64_t sites, int per) { return (sites + per * BLOCK - 1) / (per * BLOCK); }
 
 // L2 prefetch hint: `bytes` (a multiple of 16) from a 16-byte aligned address.
 __device__ __forceinline__ void l2_prefetch(const void* q, uint32_t bytes) {
@@ -965,7 +965,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 }
 
 // The sums of a state in two launches.  k_sums: blocks [0, nmass) write the
-// sums of drho (mass - sites) over kMassSites x 256 sites of [lo, hi) each into
+// sums of drho (mass - sites) over `per` x 256 sites of [lo, hi) each into
 // part[block]; in the A-B scheme the blocks after them take 256 link records
 // each and write the mass that each link lets in, recomputed from the
 // post-collision state s'(t-1), into lflux (the AA steps record it there
@@ -977,7 +977,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 template <typename S, int MODE, bool CT, bool MON>
 __global__ void __launch_bounds__(BLOCK) k_sums(const S* __restrict__ fin, const IndexTables ix,
                                                 const LinkRec* __restrict__ links, const double* __restrict__ amp,
-                                                const StepParams p, int64_t lo, int64_t hi, unsigned nmass,
+                                                const StepParams p, int64_t lo, int64_t hi, int per, unsigned nmass,
                                                 unsigned nflux, int64_t nlinks, int64_t nlist,
                                                 const int32_t* __restrict__ ilist, double* __restrict__ part,
                                                 double* __restrict__ lflux, double* __restrict__ msite) {
@@ -986,9 +986,9 @@ __global__ void __launch_bounds__(BLOCK) k_sums(const S* __restrict__ fin, const
   if (blockIdx.x < nmass) {
     __shared__ double sh[BLOCK / 32];
     double d = 0;
-    const int64_t x0 = lo + (int64_t)blockIdx.x * (kMassSites * BLOCK) + threadIdx.x;
+    const int64_t x0 = lo + (int64_t)blockIdx.x * (per * BLOCK) + threadIdx.x;
 #pragma unroll 1
-    for (int k = 0; k < kMassSites; ++k) {
+    for (int k = 0; k < per; ++k) {
       const int64_t x = x0 + k * BLOCK;
       if (x >= hi) break;
       R h[Q];
@@ -1317,10 +1317,11 @@ struct InitOp {
 template <typename S, int MODE, bool CT>
 void launch_sums(const hlb_solver* h, const S* fin, const StepParams& p, bool links, bool monitor, cudaStream_t s) {
   const int64_t lo = h->owned_lo, hi = h->owned_hi;
-  const unsigned nmass = (unsigned)mass_blocks(hi - lo), nflux = links ? grid_for(h->n_links) : 0u;
+  const int per = mass_sites(h->n);
+  const unsigned nmass = (unsigned)mass_blocks(hi - lo, per), nflux = links ? grid_for(h->n_links) : 0u;
   const unsigned nmon = monitor ? grid_for(h->n_ilist) : 0u;
   (monitor ? k_sums<S, MODE, CT, true> : k_sums<S, MODE, CT, false>)<<<nmass + nflux + nmon, BLOCK, 0, s>>>(
-      fin, h->index(), h->d_links, h->d_amp, p, lo, hi, nmass, nflux, h->n_links, h->n_ilist, h->d_ilist, h->d_red,
+      fin, h->index(), h->d_links, h->d_amp, p, lo, hi, per, nmass, nflux, h->n_links, h->n_ilist, h->d_ilist, h->d_red,
       h->d_lflux, h->d_msite);
 }
 
@@ -1337,18 +1338,19 @@ struct ReduceOp {
     const int K = h->n_iolets;
     const int64_t* begin = (const int64_t*)(h->d_red + hlb_reduce_partials(h->n));  // link ranges stored after the partials
     k_sums_finish<<<(unsigned)(monitor ? 1 + 2 * K : 1 + K), 512, 0, s>>>(
-        h->d_red, mass_blocks(owned), owned, K, h->d_lflux, begin, have_flux ? 1 : 0, h->d_msite, h->d_ioff, out, h->d_mon);
+        h->d_red, mass_blocks(owned, mass_sites(h->n)), owned, K, h->d_lflux, begin, have_flux ? 1 : 0, h->d_msite, h->d_ioff, out, out + 1 + K);
     return cudaGetLastError();
   }
 };
 
 }  // namespace
 
-int64_t hlb_reduce_partials(int64_t n) { return mass_blocks(n); }
+int64_t hlb_reduce_partials(int64_t n) { return mass_blocks(n, mass_sites(n)); }
 
 int64_t hlb_reduce_slots(int64_t n, int32_t n_iolets) {
-  // per-block partials, iolet link ranges (int64, n_iolets + 1), final outputs (1 + n_iolets)
-  return mass_blocks(n) + (n_iolets + 1) + (1 + n_iolets);
+  // per-block partials, iolet link ranges (int64, n_iolets + 1), final outputs: mass and
+  // fluxes (1 + n_iolets), monitor (2 n_iolets)
+  return hlb_reduce_partials(n) + (n_iolets + 1) + (1 + 3 * (int64_t)n_iolets);
 }
 
 cudaError_t hlb_launch_step(const hlb_solver* h, const void* fin, void* fout, bool gather, int64_t tb,

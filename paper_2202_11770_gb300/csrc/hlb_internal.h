@@ -80,7 +80,6 @@ struct hlb_solver {
   int64_t* d_ioff = nullptr;          // [n_iolets + 1] ranges of d_ilist per iolet
   int32_t* d_ilist = nullptr;         // sites with a link to iolet k, ascending, iolet by iolet
   double* d_msite = nullptr;          // [n_ilist][2] |u|^2 and rho of the sites of d_ilist (monitor scratch)
-  double* d_mon = nullptr;            // [2][n_iolets] monitor outputs
   // Windkessel outlets: host flags, device parameters, model state and the
   // ghost densities the kernels read (io_val)
   std::vector<int> wk_on;             // per iolet
@@ -195,7 +194,8 @@ cudaError_t hlb_launch_ctab(const hlb_solver* h, int32_t* misfit, cudaStream_t s
 // Equilibrium initialisation; u0 [3][n] device or null.
 cudaError_t hlb_launch_init(const hlb_solver* h, void* f, double rho0, const float* u0, cudaStream_t s);
 // Mass (out[0]) and per-iolet flux (out[1..]) in FP64; with `monitor` also
-// d_mon: per iolet max |u| (k) and mean rho (K + k) over the sites linked to it.
+// after them per iolet max |u| (out[1 + K + k]) and mean rho (out[1 + 2 K + k])
+// over the sites linked to it.
 cudaError_t hlb_launch_reduce(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux, bool monitor,
                               double* out_dev, cudaStream_t s);
 int64_t hlb_reduce_slots(int64_t n, int32_t n_iolets);

@@ -43,17 +43,17 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return r;
 }
 
-// One partial per block of kMassSites x 256 sites: sum over its sites of sum_i
+// One partial per block of `per` x 256 sites: sum over its sites of sum_i
 // h_i, as the workspace reduction (k_sums) takes it.
 template <typename S>
-__global__ void __launch_bounds__(BLOCK) k_mass_static(const S* __restrict__ f, int64_t n,
+__global__ void __launch_bounds__(BLOCK) k_mass_static(const S* __restrict__ f, int64_t n, int per,
                                                        double* __restrict__ part) {
   using R = typename Real<S>::type;
   __shared__ double sh[BLOCK / 32];
-  const int64_t x0 = (int64_t)blockIdx.x * (kMassSites * BLOCK) + threadIdx.x;
+  const int64_t x0 = (int64_t)blockIdx.x * (per * BLOCK) + threadIdx.x;
   double d = 0;
 #pragma unroll 1
-  for (int k = 0; k < kMassSites; ++k) {
+  for (int k = 0; k < per; ++k) {
     const int64_t x = x0 + k * BLOCK;
     if (x >= n) break;
     R h[Q];
@@ -100,8 +100,9 @@ int partials_address(double** out) {
 
 template <typename S>
 cudaError_t launch(const void* f, int64_t n, double* part, double* out, cudaStream_t st) {
-  const int64_t nb = (n + kMassSites * BLOCK - 1) / (kMassSites * BLOCK);
-  k_mass_static<S><<<(unsigned)nb, BLOCK, 0, st>>>((const S*)f, n, part);
+  const int per = mass_sites(n);
+  const int64_t nb = (n + per * BLOCK - 1) / (per * BLOCK);
+  k_mass_static<S><<<(unsigned)nb, BLOCK, 0, st>>>((const S*)f, n, per, part);
   k_mass_static_finish<<<1, 1024, 0, st>>>(part, nb, n, out);
   return cudaGetLastError();
 }
