@@ -230,14 +230,20 @@ __device__ __forceinline__ R cdotu(int i, R ux, R uy, R uz) {
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// Sums of products, whose two products the compiler may contract either way.
-// In FP64 its choice differed between kernels, so there the fused operations are
-// written out: every path gives the same bits.
-__device__ __forceinline__ float dot3(float ax, float ay, float az, float bx, float by, float bz) {
-  return ax * bx + ay * by + az * bz;
+// Sums of products, whose products the compiler may contract either way.  Its
+// choice differed between kernels, so the boundary values write the fused
+// operations out: every path gives the same bits.
+__device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double fmul(double a, double b) { return __dmul_rn(a, b); }
+template <typename R>
+__device__ __forceinline__ R dot3(R ax, R ay, R az, R bx, R by, R bz) {
+  return fmadd(az, bz, fmadd(ax, bx, fmul(ay, by)));
 }
-__device__ __forceinline__ double dot3(double ax, double ay, double az, double bx, double by, double bz) {
-  return fmadd(az, bz, fmadd(ay, by, ax * bx));
+// Ghost value w (drho + rho (3 cu + 4.5 cu^2 - 1.5 u.u)) of a pressure iolet.
+template <typename R>
+__device__ __forceinline__ R ghost_heq(R w, R drho, R cu, R uu) {
+  const R t = fmadd(R(3), cu, fmul(fmul(R(4.5), cu), cu));
+  return fmul(w, fmadd(R(1) + drho, fmadd(R(-1.5), uu, t), drho));
 }
 // 3 cu + 4.5 cu^2 - usq15 and the shifted equilibrium w (drho + rho b)
 __device__ __forceinline__ float heq_of(float w, float drho, float rho, float cu, float usq15) {
@@ -424,8 +430,7 @@ __device__ __forceinline__ void iolet_fixup(const S* __restrict__ fin, const int
         gz = un * BC<R>::nz(iop);
       }
       R drho = BC<R>::val(p, L.iolet);
-      R usq15 = R(1.5) * dot3(gx, gy, gz, gx, gy, gz);
-      h[i] = heq<R>(i, drho, R(1) + drho, gx, gy, gz, usq15);
+      h[i] = ghost_heq<R>(wgt<R>(i), drho, cdotu<R>(i, gx, gy, gz), dot3(gx, gy, gz, gx, gy, gz));
     }
   }
 }
@@ -492,8 +497,7 @@ __device__ __forceinline__ R lane_iolet_value(int i, const LinkRec& L, R out, R 
     gz = un * BC<R>::nz(iop);
   }
   R drho = val;
-  R usq15 = R(1.5) * dot3(gx, gy, gz, gx, gy, gz);
-  return lane_heq<R>(i, drho, R(1) + drho, gx, gy, gz, usq15);
+  return ghost_heq<R>(lane_w<R>(i), drho, lane_cdotu<R>(i, gx, gy, gz), dot3(gx, gy, gz, gx, gy, gz));
 }
 
 // ---------------------------------------------------------------------------

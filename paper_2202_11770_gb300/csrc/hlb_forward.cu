@@ -512,8 +512,7 @@ __device__ __forceinline__ R iolet_value(int i, const LinkRec& L, R out, R rho, 
     gz = un * BC<R>::nz(io);
   }
   R drho = BC<R>::val(p, L.iolet);
-  R usq15 = R(1.5) * dot3(gx, gy, gz, gx, gy, gz);
-  return heq<R>(i, drho, R(1) + drho, gx, gy, gz, usq15);
+  return ghost_heq<R>(wgt<R>(i), drho, cdotu<R>(i, gx, gy, gz), dot3(gx, gy, gz, gx, gy, gz));
 }
 
 // After an AA step at time t: overwrite the slots that the iolet links of

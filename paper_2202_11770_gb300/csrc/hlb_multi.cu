@@ -228,7 +228,12 @@ __device__ __forceinline__ void iolet_block(const S* in, S* out, const MultiArgs
         L.coef = coef[e];
         L.coef_f = (float)coef[e];
         h[e] = lane_iolet_value<R>(e * W + hl, L, o, rho_s, ux, uy, uz, amp[e], val, p);
-        if (coupled && live && k > 0) Word<double>::store(a.flux + 2 * (int64_t)(-c[e] - 2), (double)h[e] - (double)o, tag);
+        if (coupled && live && k > 0) {
+          // the outflow as k_wk_update takes it, its velocity by the reciprocal
+          const R inv = R(1) / rho_s;
+          const R m = lane_iolet_value<R>(e * W + hl, L, o, rho_s, jx * inv, jy * inv, jz * inv, amp[e], val, p);
+          Word<double>::store(a.flux + 2 * (int64_t)(-c[e] - 2), (double)m - (double)o, tag);
+        }
       }
     R drho = __shfl_sync(FULL_MASK, h[0], 0, W), cjx = R(0), cjy = R(0), cjz = R(0);
 #pragma unroll
