@@ -7,9 +7,10 @@ with a parabolic cross-section weight, rho = 1 at every outlet.  Inputs are
 synthetic and seeded; the paper's patient geometries are not available.
 
 One benchmark step = one LB time step over the whole lattice: one launch of
-the fused stream-collide-boundary kernel (pull A-B: k_step, iolet sites
-included), or for the AA pattern k_aa_odd / k_aa_even (alternating) plus
-the k_aa_fix pass over the iolet sites (0.3 % of the sites).  ``value`` is MLUPS (Eq. 9 of arXiv
+the fused stream-collide-boundary kernel (pull A-B: k_step2, iolet sites
+included), or for the AA pattern k_aa_odd2 / k_aa_even (alternating), plus on
+a lattice of this size the k_aa_fix pass over the iolet sites (0.3 % of the
+sites).  ``value`` is MLUPS (Eq. 9 of arXiv
 2202.11770) with the lattice resident in HBM, timed with one CUDA event pair
 around all timed steps; the state (~3.4 GB touched per step) is far larger
 than L2, so no flush is needed between steps.
@@ -54,18 +55,20 @@ def workload_name(n, tau):
     return (f"seeded depth-6 vessel tree, {n / 1e6:.0f}M fluid sites, D3Q19 LBGK tau={tau:g}, "
             "pulsatile Ladd inlet, 64 pressure outlets")
 
-# Index bytes per site: the int32 streaming-index table (18 x 4 B), or its
-# compact form (18 x 2 B of offsets plus 20 int32 tile bases per 256 sites).
-INDEX_BYTES = {False: 18 * 4, True: 18 * 2 + 20 * 4 / 256}
+# Index bytes per site: the int32 streaming-index table (18 x 4 B), the compact
+# table's offset form (18 x 2 B of offsets plus 20 int32 tile bases per 256
+# sites), or its row form ("rows": a mask word, 8 x 1 B of offsets and 8 int32
+# tile bases per 256 sites), which all but 2 % of the benchmark tree's tiles have.
+INDEX_BYTES = {False: 18 * 4, True: 18 * 2 + 20 * 4 / 256, "rows": 4 + 8 + 8 * 4 / 256}
 
 
 # Algorithmic bytes per site update (storage element size e): 19 populations
 # read + 19 written, plus the index table when the kernel gathers through
 # it.  Pull A-B gathers every step; the AA pattern only on odd steps.
 # Boundary-link records are O(boundary sites), not counted.
-def bytes_per_site(elem: int, kernel: str = "ab", compact: bool = False) -> float:
+def bytes_per_site(elem: int, kernel: str = "ab", compact=False) -> float:
     local = 19 * elem * 2
-    idx = INDEX_BYTES[bool(compact)]
+    idx = INDEX_BYTES[compact if compact == "rows" else bool(compact)]
     if kernel in ("ab", "aa_odd"):
         return local + idx
     if kernel == "aa_even":
@@ -232,7 +235,8 @@ def kernel_names(n, compact=True, wide=False):
 
 def form_stats(lat, precision, scheme, total, durs, t_first, steps, peak, compact):
     """MLUPS, algorithmic GB/s and per-kernel rooflines of one timed form
-    (CUDA events around every step: each step is one kernel launch)."""
+    (CUDA events around every step: each step is one kernel launch).
+    compact: False, True (offset form) or "rows" (row form of the table)."""
     n = lat.n
     k_ab, k_odd = kernel_names(n, compact)
     e = ELEM[precision]
@@ -620,7 +624,7 @@ def run_ours(args):
     clk = clocks.stop()
     ms, total_updates = aggregate_ranks(ms, n * args.steps, dist, "cuda")
     value = total_updates / (ms * 1e-3) / 1e6
-    head = form_stats(lat, prec0, scheme, ms, durs, t_first, args.steps, peak, compact)
+    head = form_stats(lat, prec0, scheme, ms, durs, t_first, args.steps, peak, "rows" if compact else False)
     kname = kernel_names(n, compact, args.wide_offsets)[0 if scheme == "ab" else 1]
     kst = head["kernels"][kname]
     traffic = None
@@ -639,7 +643,7 @@ def run_ours(args):
                     continue
                 tot, d, tf, ct = time_form(lat, prec, sch, args.steps, args.warmup, torch, dist,
                                            full_index=args.full_index)
-                forms[f"{prec}_{sch}"] = form_stats(lat, prec, sch, tot, d, tf, args.steps, peak, ct)
+                forms[f"{prec}_{sch}"] = form_stats(lat, prec, sch, tot, d, tf, args.steps, peak, "rows" if ct else False)
 
     adjoint = None
     if not args.quick and args.adjoint_steps > 0:
@@ -671,21 +675,24 @@ def run_ours(args):
             "vs_baseline": None, "dtype": {"fp32": "f32", "bf16": "bf16 storage, f32 math", "fp16": "f16 storage, f32 math", "fp64": "f64"}[prec0], "data": "synthetic",
             "config": {"workload": workload_name(n, args.tau), "n_sites": n, "tau": args.tau,
                        "scheme": {"ab": "pull A-B", "aa": "AA pattern"}[scheme],
-                       "index": ("compact: 16-bit offsets from per-tile bases" if compact else "int32 table"),
+                       "index": ("compact: link mask and 8-bit row offsets from per-tile bases" if compact else "int32 table"),
                        "parallelism": f"replicas x{world}", "l2": f"working set {n * head['bytes_per_site'] / 1e9:.1f} GB/step >> 129 MB L2, no flush",
                        "fill": round(lat.info["fill"], 4)},
             "roofline": {"bound": "hbm", "achieved": kst["gbs"], "peak": peak, "unit": "GB/s",
                          "frac": kst["gbs"] / peak, "traffic": traffic, "peak_kind": peak_kind,
-                         "kernel": f"{kname}<{CTYPE[prec0]}>", "launches": kst["launches"], "mean_us": kst["mean_us"],
+                         # FP32 and 16-bit storage on the compact table: the two-site kernels
+                         "kernel": (f"{kname.rstrip('2')}{'2' if compact and ELEM[prec0] <= 4 else ''}"
+                                    f"<{CTYPE[prec0]}>"), "launches": kst["launches"], "mean_us": kst["mean_us"],
                          "timed": "CUDA events around each step" + (
-                             " (odd step = k_aa_odd + the k_aa_fix pass)" if scheme == "aa" else ""),
+                             " (odd step = the kernel + the k_aa_fix pass)" if scheme == "aa" else ""),
                          "algorithmic_bytes_per_site": kst["bytes_per_site"],
                          "step_gbs": head["gbs"], "step_bytes_per_site": head["bytes_per_site"]},
             "cpu_baseline": cpu,
             "e2e": e2e,
             "clocks": clk,
-            # per step: the fused kernel, plus the iolet fix-up pass for AA
-            "gpu_launches": args.steps * (2 if scheme == "aa" and bool((lat.src <= -2).any()) else 1),
+            # per step: the fused kernel, plus the iolet pass of an AA step on a large lattice
+            "gpu_launches": args.steps * (2 if scheme == "aa" and bool((lat.src <= -2).any()) and not (
+                compact and prec0 == "fp32" and n < 4_000_000) else 1),
             "forms": forms,
             "precision_vs_oracle": precision,
             "adjoint": adjoint,

@@ -487,6 +487,9 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   for (const LinkRef& l : links) isites.push_back(l.x);
   std::sort(isites.begin(), isites.end());
   isites.erase(std::unique(isites.begin(), isites.end()), isites.end());
+  h->spread_sites = (n + hlb::kSpread * 512 - 1) / (hlb::kSpread * 512) * 512;
+  for (int k = 0; k <= hlb::kSpread; ++k)
+    h->spread_count.push_back(std::lower_bound(isites.begin(), isites.end(), std::min<int64_t>(n, k * h->spread_sites)) - isites.begin());
   cudaError_t e = cudaSuccess;
   // the caller's rows straight into the padded device table (no host copy of
   // the table), padding entries (never gathered) -1, then the iolet links

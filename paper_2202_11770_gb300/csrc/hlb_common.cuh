@@ -151,6 +151,33 @@ __device__ __forceinline__ uint32_t block_div(uint32_t b, const BlockDiv& q) {
   return q.m == 0 ? (b >> q.s) : (__umulhi(b, q.m) >> q.s);
 }
 
+// How the iolet blocks of a step's grid lie among its bulk blocks.  The site
+// list is cut into kSpread segments; the blocks of segment s are the grid's
+// blocks [blk[s], blk[s + 1]), of which the iolet blocks number io[s] ..
+// io[s + 1] - 1, evenly spaced.  An iolet site so runs at about the time that
+// its neighbours in memory do: its 4 (2) bytes of a 32-byte sector join theirs
+// in L2, where the same blocks spread over the whole grid wrote the sector to
+// DRAM twice.  Block r of a segment is an iolet block when floor(r k / 2^32)
+// steps from r to r + 1, k = ceil(2^32 iolet blocks / blocks).  segments = 1:
+// the whole grid is segment 0 (no search).
+constexpr int kSpread = 64;
+struct IoletSpread {
+  uint32_t segments, blk[kSpread + 1], io[kSpread + 1], k[kSpread];
+};
+// True for an iolet block, *number its number; else *number the bulk block's.
+__device__ __forceinline__ bool spread_block(const IoletSpread& sp, uint32_t b, uint32_t* number) {
+  int s = 0;
+  if (sp.segments > 1) {
+#pragma unroll
+    for (int step = kSpread / 2; step > 0; step >>= 1)
+      if (sp.blk[s + step] <= b) s += step;
+  }
+  const uint32_t r = b - sp.blk[s], before = __umulhi(r, sp.k[s]);
+  const bool iolet = __umulhi(r + 1, sp.k[s]) != before;
+  *number = iolet ? sp.io[s] + before : b - sp.io[s] - before;
+  return iolet;
+}
+
 // Relaxation rate 1/tau in the arithmetic type of a kernel.
 template <typename R> __device__ __forceinline__ R omega_of(const StepParams& p);
 template <> __device__ __forceinline__ float omega_of<float>(const StepParams& p) { return p.omegaf; }

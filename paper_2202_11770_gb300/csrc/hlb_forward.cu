@@ -10,7 +10,7 @@
 //  * pull A-B (k_step, k_step2): read buffer A by gathering through the index
 //    table, write buffer B; 164 B per FP32 site update with the row form of
 //    the compact index table (224 B with the int32 one).
-//  * AA pattern (k_aa_even / k_aa_odd, then k_aa_fix over iolet sites): one
+//  * AA pattern (k_aa_even / k_aa_odd and their two-site forms): one
 //    buffer.  Even steps read a site's 19 slots and write them back swapped
 //    (no index table); odd steps read 19 slots through the index table and
 //    write the results to the very same 19 slots.  152 B (even) + 164 B
@@ -45,7 +45,7 @@ template <typename S> constexpr int pair_blocks() { return sizeof(S) == 4 ? 6 : 
 // Lanes a site in the AA iolet pass (8 lanes 1-2 us slower a step on the
 // 20M-site tree, 32 lanes 3 us slower).
 constexpr int kFixLanes = 16;
-
+constexpr uint32_t kNoTile = 0xffffffffu;  // first tile of a launch without tiles
 constexpr int READ = 128;  // threads a block of the read-back kernels, one site each
 
 inline unsigned grid_for(int64_t n) { return (unsigned)((n + BLOCK - 1) / BLOCK); }
@@ -199,18 +199,19 @@ template <typename S, bool WIDE, bool CT>
 __global__ void __launch_bounds__(BLOCK, 5) k_step(const S* __restrict__ fin, S* __restrict__ fout,
                                                 const IndexTables ix, const LinkRec* __restrict__ links,
                                                 const double* __restrict__ amp, const int32_t* __restrict__ sites,
-                                                int64_t nsites, unsigned n_iolet_blocks, const BlockDiv stride,
-                                                uint32_t pf, uint32_t tile0, const StepParams p) {
+                                                int64_t nsites, const IoletSpread spread, uint32_t pf, uint32_t tile0,
+                                                const StepParams p) {
   using R = typename Real<S>::type;
-  const unsigned b = blockIdx.x, j = block_div(b, stride);
-  if (b == j * stride.d && j < n_iolet_blocks) {
+  uint32_t j;
+  if (spread_block(spread, blockIdx.x, &j)) {
     pdl_wait();
     pdl_trigger();
     step_iolet_site<S>(fin, fout, ix.src, links, amp, sites, nsites, p, ((int64_t)j * BLOCK + threadIdx.x) / kStepIoletLanes);
     return;
   }
   const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
-  const uint32_t tile = tile0 + b - min(n_iolet_blocks, j + 1);
+  if (tile0 == kNoTile) return;
+  const uint32_t tile = tile0 + j;
   const uint32_t x = tile * BLOCK + threadIdx.x;
   if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, false>(fin, ix, n, sn, tile + pf);
   uint32_t off[Q];
@@ -240,15 +241,146 @@ __global__ void __launch_bounds__(BLOCK, 5) k_step(const S* __restrict__ fin, S*
 // ---------------------------------------------------------------------------
 // AA pattern.
 // ---------------------------------------------------------------------------
-// Even step: f(t) in place -> collide -> s'(t) stored swapped (slot ibar).
-template <typename S>
-__global__ void __launch_bounds__(BLOCK) k_aa_even(S* A, const StepParams p) {
+// The sites with iolet links of an AA step at time t, W lanes a site, lane h
+// holding directions h, h + W, ...: f(t) from the slots (EVEN: the site's own,
+// ODD: through its codes), collision, and each post-collision population into
+// the slot that its opposite direction was read from.  An iolet link's slot
+// (slot i of x in both parities) gets the boundary value that the next step
+// reads instead, from the moments of the stored (rounded) post-collision
+// populations as the A-B gather takes them, and the mass that the link lets
+// in is recorded.  No other site touches these slots, so the sites can be blocks
+// of the step's own grid, every stride-th one, instead of a pass of their own
+// after each step (k_aa_fix): aa_in_grid says when.  Codes, records and
+// amplitudes load before the wait for the previous step; icode holds a site's
+// 18 codes contiguously.
+template <typename S, bool ODD>
+__device__ __forceinline__ void aa_iolet_site(S* A, const int32_t* __restrict__ icode, const LinkRec* __restrict__ links,
+                                              const double* __restrict__ amp, const int32_t* __restrict__ sites,
+                                              int64_t nsites, const StepParams& p, double* __restrict__ lflux, int64_t q0) {
   using R = typename Real<S>::type;
-  const int64_t n = p.n;
-  const int64_t x = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
+  constexpr int W = kStepIoletLanes, NE = (Q + W - 1) / W;
+  const bool live = q0 < nsites;
+  const int64_t q = live ? q0 : 0, n = p.n;  // lanes past the end shadow site 0 and store nothing
+  const int hl = threadIdx.x & (W - 1);
+  const int64_t x = __ldg(sites + q);
+  int32_t c[NE];
+  LinkRec L[NE];
+  R a[NE], h[NE];
+#pragma unroll
+  for (int e = 0; e < NE; ++e) {
+    const int i = e * W + hl;
+    c[e] = (i >= 1 && i < Q) ? __ldg(icode + q * (Q - 1) + (i - 1)) : 0;
+    L[e] = links[c[e] <= -2 ? -c[e] - 2 : 0];  // record 0 exists whenever there are iolet sites
+    a[e] = BC<R>::amp(p, amp, L[e].kind == 0 && L[e].group >= 0 ? L[e].group : 0);
+  }
   pdl_wait();
   pdl_trigger();
-  if (x >= n) return;
+#pragma unroll
+  for (int e = 0; e < NE; ++e) {
+    const int i = e * W + hl;
+    h[e] = i < Q ? to_real(A[i == 0 ? x : (ODD ? aa_addr(i, c[e], n, x) : (int64_t)i * n + x)]) : R(0);
+  }
+  auto in = [&](int k) { return __shfl_sync(FULL_MASK, h[k / W], k % W, W); };
+  R o[NE];  // s'_i(x), as stored
+  {
+    R drho = in(0), jx = R(0), jy = R(0), jz = R(0);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const int ip = 2 * k + 1;
+      const R va = in(ip), vb = in(ip + 1), dp = va - vb;
+      drho += va + vb;
+      if (cx(ip)) jx = cx(ip) > 0 ? jx + dp : jx - dp;
+      if (cy(ip)) jy = cy(ip) > 0 ? jy + dp : jy - dp;
+      if (cz(ip)) jz = cz(ip) > 0 ? jz + dp : jz - dp;
+    }
+    const Bgk<R> b(drho, jx, jy, jz, omega_of<R>(p));
+#pragma unroll
+    for (int e = 0; e < NE; ++e) o[e] = e * W + hl < Q ? to_real(from_real<S>(iolet_lane_out<R>(e * W + hl, h[e], b))) : R(0);
+  }
+  // rho = 1 + sum s'_k, j = sum s'_k c_k in direction order
+  R d = R(0), jx = R(0), jy = R(0), jz = R(0);
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    const R vk = __shfl_sync(FULL_MASK, o[k / W], k % W, W);
+    d += vk;
+    if (cx(k)) jx += cx(k) > 0 ? vk : -vk;
+    if (cy(k)) jy += cy(k) > 0 ? vk : -vk;
+    if (cz(k)) jz += cz(k) > 0 ? vk : -vk;
+  }
+  const R rho = R(1) + d;
+  const R ux = jx / rho, uy = jy / rho, uz = jz / rho;
+  // s'_opp(i): direction i + 1 for odd i (odd lanes, W even), i - 1 for even i
+  R up[NE + 1], dn[NE + 1];
+#pragma unroll
+  for (int e = 0; e < NE; ++e) {
+    up[e] = __shfl_sync(FULL_MASK, o[e], (hl + 1) & (W - 1), W);
+    dn[e + 1] = __shfl_sync(FULL_MASK, o[e], (hl + W - 1) & (W - 1), W);
+  }
+  up[NE] = dn[0] = R(0);
+  if (!live) return;
+#pragma unroll
+  for (int e = 0; e < NE; ++e) {
+    const int i = e * W + hl;
+    if (i >= Q) continue;
+    if (i == 0) {
+      stpop<S>(A + x, o[0]);
+      continue;
+    }
+    R v = (i & 1) ? (hl == W - 1 ? up[e + 1] : up[e]) : (hl == 0 ? dn[e] : dn[e + 1]);
+    if (c[e] <= -2) {
+      const R val = lane_iolet_value<R>(i, L[e], v, rho, ux, uy, uz, a[e], BC<R>::val(p, L[e].iolet), p);
+      lflux[-c[e] - 2] = (double)val - (double)v;
+      v = val;
+    }
+    stpop<S>(A + (ODD ? aa_addr(i, c[e], n, x) : (int64_t)i * n + x), v);
+  }
+}
+
+// The iolet blocks of an AA step's grid (GRID; otherwise the bulk blocks take
+// all sites and k_aa_fix follows).
+struct AAIolets {
+  const int32_t* icode;
+  const LinkRec* links;
+  const double* amp;
+  const int32_t* sites;
+  int64_t nsites;
+  const uint32_t* imask;
+  double* lflux;
+  unsigned blocks;  // iolet blocks, every stride-th of the grid's first ones
+  BlockDiv stride;
+};
+// True for an iolet block, whose sites it steps; otherwise *bulk is the bulk block's number.
+template <typename S, bool ODD, bool GRID>
+__device__ __forceinline__ bool aa_iolet_block(S* A, const AAIolets& io, const StepParams& p, uint32_t* bulk) {
+  if (!GRID) {
+    *bulk = blockIdx.x;
+    return false;
+  }
+  const unsigned b = blockIdx.x, j = block_div(b, io.stride);
+  *bulk = b - min(io.blocks, j + 1);
+  if (b != j * io.stride.d || j >= io.blocks) return false;
+  aa_iolet_site<S, ODD>(A, io.icode, io.links, io.amp, io.sites, io.nsites, p, io.lflux,
+                               ((int64_t)j * blockDim.x + threadIdx.x) / kStepIoletLanes);
+  return true;
+}
+// Whether the iolet blocks step site x.
+template <bool GRID>
+__device__ __forceinline__ bool left_to_iolets(const AAIolets& io, uint32_t x) {
+  return GRID && ((__ldg(io.imask + (x >> 5)) >> (x & 31)) & 1u);
+}
+
+// Even step: f(t) in place -> collide -> s'(t) stored swapped (slot ibar).
+template <typename S, bool GRID>
+__global__ void __launch_bounds__(BLOCK) k_aa_even(S* A, const AAIolets io, const StepParams p) {
+  using R = typename Real<S>::type;
+  uint32_t bulk;
+  if (aa_iolet_block<S, false, GRID>(A, io, p, &bulk)) return;
+  const int64_t n = p.n;
+  const int64_t x = (int64_t)bulk * BLOCK + threadIdx.x;
+  const bool skip = x >= n || left_to_iolets<GRID>(io, (uint32_t)x);
+  pdl_wait();
+  pdl_trigger();
+  if (skip) return;
   R h[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) h[i] = to_real(A[(int64_t)i * n + x]);
@@ -436,17 +568,18 @@ template <typename S, bool WIDE>
 __global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_step2(const S* __restrict__ fin, S* __restrict__ fout,
                                                 const IndexTables ix, const LinkRec* __restrict__ links,
                                                 const double* __restrict__ amp, const int32_t* __restrict__ sites,
-                                                int64_t nsites, unsigned n_iolet_blocks, const BlockDiv stride,
-                                                uint32_t pf, uint32_t tile0, const StepParams p) {
-  const unsigned b = blockIdx.x, j = block_div(b, stride);
-  if (b == j * stride.d && j < n_iolet_blocks) {
+                                                int64_t nsites, const IoletSpread spread, uint32_t pf, uint32_t tile0,
+                                                const StepParams p) {
+  uint32_t j;
+  if (spread_block(spread, blockIdx.x, &j)) {
     pdl_wait();
     pdl_trigger();
     step_iolet_site<S>(fin, fout, ix.src, links, amp, sites, nsites, p, ((int64_t)j * PAIR + threadIdx.x) / kStepIoletLanes);
     return;
   }
   const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
-  const uint32_t tile = tile0 + b - min(n_iolet_blocks, j + 1);
+  if (tile0 == kNoTile) return;
+  const uint32_t tile = tile0 + j;
   const uint32_t x = pair_site(tile), y = x + 32;
   if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, false>(fin, ix, n, sn, tile + pf);
   int32_t bs[CT_GROUPS];
@@ -594,7 +727,7 @@ __global__ void __launch_bounds__(256, 8) k_aa_fix(S* A, const int32_t* __restri
 // Odd step: gather f(t) through the index table, collide, and write each
 // post-collision population into the slot it came from, where the site
 // downstream (or, across a wall or iolet, the site itself) reads it in the
-// next (even) step.  Iolet links get their boundary values from k_aa_fix.
+// next (even) step.  Sites with iolet links: aa_iolet_site or k_aa_fix.
 // This one-site form serves FP64 storage and the int32 table; k_aa_odd2 the
 // rest.  The 18 slot offsets (32-bit) are computed once and held in registers
 // for the stores, so the index row is read once.  WIDE: offsets within
@@ -635,21 +768,24 @@ __global__ void __launch_bounds__(BLOCK, WIDE ? 4 : 5) k_aa_odd(S* A, const Inde
 // lets two sites share a thread at 80 (72) registers.  20M-site tree, step
 // with the iolet pass: FP32 597 -> 532 us, BF16 460 -> 388 us; 2.0M sites FP32
 // 75 -> 67, BF16 58 -> 48 us.
-template <typename S, bool WIDE>
-__global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_aa_odd2(S* A, const IndexTables ix, uint32_t pf,
-                                                               const StepParams p) {
-  const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn, tile = blockIdx.x;
+template <typename S, bool WIDE, bool GRID>
+__global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_aa_odd2(S* A, const IndexTables ix, const AAIolets io, uint32_t pf,
+                                                                        const StepParams p) {
+  uint32_t tile;
+  if (aa_iolet_block<S, true, GRID>(A, io, p, &tile)) return;
+  const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
   const uint32_t x = pair_site(tile), y = x + 32;
   if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, true>(A, ix, n, sn, tile + pf);
   int32_t bs[CT_GROUPS];
   if (load_row_bases(ix, tile, bs)) {
-    const bool two = y < n;
-    const uint32_t y1 = two ? y : x;  // a thread without a second site repeats its first, and does not store it
+    const uint32_t y1 = y < n ? y : x;  // a thread without a second site repeats its first, and does not store it
     uint32_t wa[CT_ROW_WORDS], wb[CT_ROW_WORDS];
     if (x < n) load_pair_words(ix, WIDE, sn, x, y1, wa, wb);
     pdl_wait();
     pdl_trigger();
     if (x >= n) return;
+    constexpr uint32_t iolet = GRID ? 1u << CT_IOLET_BIT : 0u;
+    const bool da = !(wa[0] & iolet), db = y < n && !(wb[0] & iolet);
     uint32_t pa[CT_GROUPS + 1], pb[CT_GROUPS + 1];
     row_positions(x, bs, wa[1], wa[2], pa);
     row_positions(y1, bs, wb[1], wb[2], pb);
@@ -667,18 +803,19 @@ __global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_aa_odd2(S* A, const 
     load_row_bases(ix, tile, bs);
     row_positions(x, bs, wa[1], wa[2], pa);
     row_positions(y, bs, wb[1], wb[2], pb);
-    stpop<S>(A + x, o[0].x);
-    if (two) stpop<S>(A + y, o[0].y);
+    if (da) stpop<S>(A + x, o[0].x);
+    if (db) stpop<S>(A + y, o[0].y);
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-      stpop<S>(at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wa[0], pa, n)), o[opp(i)].x);
-      if (two) stpop<S>(at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wb[0], pb, n)), o[opp(i)].y);
+      if (da) stpop<S>(at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wa[0], pa, n)), o[opp(i)].x);
+      if (db) stpop<S>(at<WIDE>(A, i, n, row_offset<WIDE, true>(i, wb[0], pb, n)), o[opp(i)].y);
     }
     return;
   }
   pdl_wait();
   pdl_trigger();
   for (uint32_t z = x; z < n && z <= y; z += 32) {
+    if (left_to_iolets<GRID>(io, z)) continue;
     int32_t code[Q];
     offset_links<WIDE, LD_NC>(ix, sn, z, tile, [&](int i, bool fluid, uint32_t s) { code[i] = fluid ? (int32_t)s : -1; });
     uint32_t off[Q];
@@ -1087,30 +1224,68 @@ cudaError_t dispatch(int precision, A... a) {
   return cudaErrorInvalidValue;
 }
 
+inline unsigned iolet_blocks(const hlb_solver* h, int threads) {
+  return (unsigned)((h->n_iolet_sites * kStepIoletLanes + threads - 1) / threads);
+}
+constexpr int64_t kSpreadSites = 4000000;
+inline uint32_t spread_factor(uint32_t iolet, uint32_t blocks) {
+  return blocks ? (uint32_t)((((uint64_t)iolet << 32) + blocks - 1) / blocks) : 0u;
+}
+// The grid of a whole step with bulk blocks of `sites` sites and `threads`
+// threads, its iolet blocks among those of their own sites.  A segment's iolet
+// blocks are fewer than its blocks (its last holds the ones left over), so
+// spread_factor stays below 2^32.
+unsigned spread_iolets(const hlb_solver* h, int sites, int threads, IoletSpread* sp) {
+  const int per = threads / kStepIoletLanes;
+  const uint32_t bulk = (uint32_t)((h->n + sites - 1) / sites), all = iolet_blocks(h, threads);
+  sp->segments = kSpread;
+  for (int s = 0; s <= kSpread; ++s) {
+    const int64_t x = s * h->spread_sites;
+    const bool end = x >= h->n;
+    sp->io[s] = end ? all : (uint32_t)(h->spread_count[(size_t)s] / per);
+    sp->blk[s] = (end ? bulk : (uint32_t)(x / sites)) + sp->io[s];
+  }
+  for (int s = 0; s < kSpread; ++s) sp->k[s] = spread_factor(sp->io[s + 1] - sp->io[s], sp->blk[s + 1] - sp->blk[s]);
+  return bulk + all;
+}
+// `bulk` bulk blocks with `iolet` iolet blocks spread evenly among them.  Iolet
+// blocks alone get one bulk block, which has nothing to do (kNoTile).
+unsigned spread_evenly(uint32_t bulk, uint32_t iolet, IoletSpread* sp) {
+  if (bulk == 0 && iolet > 0) bulk = 1;
+  sp->segments = 1;
+  sp->blk[0] = sp->io[0] = 0;
+  sp->k[0] = spread_factor(iolet, bulk + iolet);
+  return bulk + iolet;
+}
+
 // One pull A-B gather step over the bulk tiles [tile0, tile0 + ntiles) and,
 // with `iolets`, the iolet sites (the whole step: tile0 = 0, all tiles).
 template <typename S>
 cudaError_t launch_gather(const hlb_solver* h, const void* fin, void* fout, const StepParams& p, uint32_t tile0,
                           uint32_t ntiles, bool iolets, cudaStream_t s) {
+  // a whole step past L2: the iolet blocks beside their sites (FP32 8.0M sites 215 -> 204 us, 20M 497 -> 483;
+  // 16 bits the same); a small lattice, or a part of the step: evenly among its tiles, which needs no search
+  // (0.5M sites, BF16: 10.0 us a step, 10.5 with it)
+  const bool whole = iolets && tile0 == 0 && ntiles == grid_for(h->n) && h->n >= kSpreadSites;
+  IoletSpread spread;
+  if (ntiles == 0) tile0 = kNoTile;
   if constexpr (sizeof(S) <= 4) {
     if (h->compact) {
-      const unsigned gi = iolets ? (unsigned)((h->n_iolet_sites * kStepIoletLanes + PAIR - 1) / PAIR) : 0u;
-      const unsigned grid = gi + ntiles;
+      const unsigned grid = whole ? spread_iolets(h, CT_TILE, PAIR, &spread)
+                                  : spread_evenly(ntiles, iolets ? iolet_blocks(h, PAIR) : 0u, &spread);
       if (grid == 0) return cudaSuccess;
       return launch_pdl(h->off32 ? k_step2<S, false> : k_step2<S, true>, grid, PAIR, s, (const S*)fin, (S*)fout, h->index(),
-                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, gi, make_block_div(gi ? grid / gi : 1),
-                        (uint32_t)h->n_sm * 3u, tile0, p);
+                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, spread, (uint32_t)h->n_sm * 3u, tile0, p);
     }
   }
-  const unsigned gi = iolets ? (unsigned)((h->n_iolet_sites * kStepIoletLanes + BLOCK - 1) / BLOCK) : 0u;
-  const unsigned grid = gi + ntiles;
+  const unsigned grid = whole ? spread_iolets(h, BLOCK, BLOCK, &spread)
+                              : spread_evenly(ntiles, iolets ? iolet_blocks(h, BLOCK) : 0u, &spread);
   if (grid == 0) return cudaSuccess;
   constexpr bool CT = sizeof(S) > 4;  // FP64 only: the others take two sites a thread
   auto kernel = h->compact ? (h->off32 ? k_step<S, false, CT> : k_step<S, true, CT>)
                            : (h->off32 ? k_step<S, false, false> : k_step<S, true, false>);
   return launch_pdl(kernel, grid, BLOCK, s, (const S*)fin, (S*)fout, h->index(), h->d_links, h->d_amp,
-                    h->d_iolet_sites, h->n_iolet_sites, gi, make_block_div(gi ? grid / gi : 1),
-                    (uint32_t)h->n_sm * 5u, tile0, p);
+                    h->d_iolet_sites, h->n_iolet_sites, spread, (uint32_t)h->n_sm * 5u, tile0, p);
 }
 
 template <typename S>
@@ -1132,46 +1307,59 @@ struct StepRangeOp {
   }
 };
 
+// Whether an AA step takes its iolet sites in its own grid or leaves them to
+// k_aa_fix.  In the grid they save a launch and its wait, but hold slots of the
+// bulk blocks while they wait for scattered loads.  Measured per step, in the
+// grid against the pass, FP32: 0.5M sites 13.0 / 15.1 us, 1.0M 23.6 / 26.4, 2.0M
+// 54.9 / 57.8, 8.0M 214 / 210, 20M 503 / 492.  16-bit storage gains less (2.0M
+// 38.6 / 38.2, 20M 345 / 312) and keeps the pass, as FP64 and the int32 table do.
 template <typename S>
-cudaError_t aa_even(const hlb_solver* h, S* A, const StepParams& p, cudaStream_t s) {
-  return launch_pdl(k_aa_even<S>, grid_for(h->n), BLOCK, s, A, p);
-}
-template <typename S>
-cudaError_t aa_even_pairs(const hlb_solver* h, S* A, const StepParams& p, cudaStream_t s) {
-  if (h->n % 2 == 0) return launch_pdl(k_aa_even2<S>, grid_for(h->n / 2), BLOCK, s, A, p);
-  return launch_pdl(k_aa_even<S>, grid_for(h->n), BLOCK, s, A, p);
-}
-template <>
-cudaError_t aa_even<__nv_bfloat16>(const hlb_solver* h, __nv_bfloat16* A, const StepParams& p, cudaStream_t s) {
-  return aa_even_pairs<__nv_bfloat16>(h, A, p, s);
-}
-template <>
-cudaError_t aa_even<__half>(const hlb_solver* h, __half* A, const StepParams& p, cudaStream_t s) {
-  return aa_even_pairs<__half>(h, A, p, s);
+bool aa_in_grid(const hlb_solver* h) {
+  return sizeof(S) == 4 && h->compact && h->n < 4000000;
 }
 
-template <typename S>
-cudaError_t aa_odd(const hlb_solver* h, S* A, const StepParams& p, cudaStream_t s) {
-  if constexpr (sizeof(S) <= 4) {
-    if (h->compact)
-      return launch_pdl(h->off32 ? k_aa_odd2<S, false> : k_aa_odd2<S, true>, grid_for(h->n), PAIR, s, A, h->index(),
-                        (uint32_t)h->n_sm * 3u, p);
+// The iolet blocks of a grid with `bulk` bulk blocks of `threads` threads.
+template <bool GRID>
+AAIolets aa_iolets(const hlb_solver* h, unsigned bulk, int threads) {
+  const unsigned gi = GRID ? iolet_blocks(h, threads) : 0u;
+  return {h->d_icode, h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, h->d_imask, h->d_lflux, gi,
+          make_block_div(gi ? (bulk + gi) / gi : 1)};
+}
+
+template <typename S, bool GRID>
+cudaError_t launch_aa(const hlb_solver* h, S* A, bool odd, const StepParams& p, cudaStream_t s) {
+  const unsigned g = grid_for(h->n);
+  if (odd) {
+    if constexpr (sizeof(S) <= 4) {
+      if (h->compact) {
+        const AAIolets io = aa_iolets<GRID>(h, g, PAIR);
+        return launch_pdl(h->off32 ? k_aa_odd2<S, false, GRID> : k_aa_odd2<S, true, GRID>, g + io.blocks, PAIR, s, A,
+                          h->index(), io, (uint32_t)h->n_sm * 3u, p);
+      }
+    }
+    if constexpr (!GRID) {
+      constexpr bool CT = sizeof(S) > 4;  // FP64 only: the others take two sites a thread
+      return launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, CT> : k_aa_odd<S, true, CT>)
+                                   : (h->off32 ? k_aa_odd<S, false, false> : k_aa_odd<S, true, false>),
+                        g, BLOCK, s, A, h->index(), (uint32_t)h->n_sm * (h->off32 ? 3u : 4u), p);
+    }
+    return cudaErrorInvalidValue;  // GRID: compact FP32
   }
-  constexpr bool CT = sizeof(S) > 4;  // FP64 only: the others take two sites a thread
-  return launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, CT> : k_aa_odd<S, true, CT>)
-                               : (h->off32 ? k_aa_odd<S, false, false> : k_aa_odd<S, true, false>),
-                    grid_for(h->n), BLOCK, s, A, h->index(), (uint32_t)h->n_sm * (h->off32 ? 3u : 4u), p);
+  if constexpr (sizeof(S) == 2) {
+    if (h->n % 2 == 0) return launch_pdl(k_aa_even2<S>, grid_for(h->n / 2), BLOCK, s, A, p);
+  }
+  const AAIolets io = aa_iolets<GRID>(h, g, BLOCK);
+  return launch_pdl(k_aa_even<S, GRID>, g + io.blocks, BLOCK, s, A, io, p);
 }
 
 template <typename S>
 struct AAOp {
   static cudaError_t run(const hlb_solver* h, void* A, bool odd, int64_t t, cudaStream_t s) {
-    StepParams p = h->params(t);
-    cudaError_t e;
-    if (odd)
-      e = aa_odd<S>(h, (S*)A, p, s);
-    else
-      e = aa_even<S>(h, (S*)A, p, s);
+    const StepParams p = h->params(t);
+    if constexpr (sizeof(S) == 4) {
+      if (aa_in_grid<S>(h)) return launch_aa<S, true>(h, (S*)A, odd, p, s);
+    }
+    const cudaError_t e = launch_aa<S, false>(h, (S*)A, odd, p, s);
     if (e != cudaSuccess || h->n_iolet_sites == 0) return e;
     constexpr int per_block = 256 / kFixLanes;  // iolet sites a block
     const unsigned g = (unsigned)((h->n_iolet_sites + per_block - 1) / per_block);

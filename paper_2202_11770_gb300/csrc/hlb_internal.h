@@ -97,6 +97,8 @@ struct hlb_solver {
     return false;
   }
   int64_t n_iolet_sites = 0;
+  int64_t spread_sites = 0;           // sites of a segment of IoletSpread (a multiple of 512)
+  std::vector<int64_t> spread_count;  // [kSpread + 1] iolet sites before each segment
   int64_t n_ilist = 0;                // entries of d_ilist
   int64_t red_slots = 0;
 
