@@ -123,10 +123,12 @@ typedef struct {
  *   lattices.  Results are identical either way.
  * full_index: 1 = the step and adjoint kernels read the 32-bit streaming
  *   index table.  By default (0) they read a compact copy built at create:
- *   per 256-site tile and direction the smallest fluid source, and per site
- *   and direction a 16-bit offset from it (36 instead of 72 bytes a site).
- *   The lattice's sources are ordered as its sites, so in a vessel lattice
- *   the sources of one direction over a tile span a few hundred sites; if
+ *   per 256-site tile a mask of each site's fluid links and eight 8-bit
+ *   offsets for the lattice rows that its sources lie in (12 instead of 72
+ *   bytes a site); a tile whose rows have holes keeps per direction its
+ *   smallest fluid source, and per site and direction a 16-bit offset from it
+ *   (36 bytes a site).  The lattice's sources are ordered as its sites, so in
+ *   a vessel lattice both fit; if
  *   some tile's span does not fit 16 bits the library uses the 32-bit table
  *   (hlb_compact_index reports which).  Results are identical either way. */
 typedef struct {
@@ -223,9 +225,11 @@ int hlb_windkessel_state(hlb_solver* h, int32_t k, double* rho_ghost, double* rh
 int hlb_init_equilibrium(hlb_solver* h, double rho0, const float* u0, int32_t where);
 
 /* Advance n >= 0 time steps (Section 3.1 steps 2-5), asynchronously: per
- * step one fused collide-stream-boundary kernel launch (pull A-B: iolet
- * sites included), plus for the AA scheme the boundary pass over the iolet
- * sites, plus one small update kernel when Windkessel outlets are set. */
+ * step one fused collide-stream-boundary kernel launch, plus, for the AA
+ * scheme on a large lattice, a boundary pass over the iolet sites, plus one
+ * small update kernel when Windkessel outlets are set.  A small lattice of the
+ * pull scheme takes all n steps (n >= 4) in one launch, or a few, outside a
+ * stream capture. */
 int hlb_step(hlb_solver* h, int64_t n);
 int hlb_time(const hlb_solver* h, int64_t* t);
 

@@ -216,13 +216,13 @@ int validate(const hlb_lattice* L, const hlb_options* o, std::vector<int64_t>* p
   return HLB_OK;
 }
 
-// AUTO resolves to the scheme measured faster on GB300 for the lattice size.
-// The AA pattern moves 170 B per FP32 site update against 188 B for pull
-// A-B (compact index table), but needs a second launch per step for its
-// iolet-site pass.  Measured per step (seeded vessel trees, FP32 / BF16):
-// 0.5M sites A-B 13.4 / 12.0 us, AA 14.8 / 12.6 us (the state fits in L2);
-// 1.0M sites A-B 32.4 / 23.8 us, AA 29.8 / 19.9 us; 2.0M 67.7 / 49.4 against
-// 61.7 / 42.3 us; 8.0M 256 / 188 against 229 / 145 us.  AA from 750k sites.
+// AUTO resolves by lattice size.  The AA pattern moves 158 B per FP32 site
+// update against 164 B for pull A-B (row-form index) and needs one buffer
+// instead of two.  Measured per step (seeded vessel trees), pull A-B / AA: FP32
+// 0.5M sites 12.7 / 13.0 us (the state fits in L2), 1.0M 29.7 / 23.6, 2.0M 56.1
+// / 54.9, 8.0M 204 / 210, 20M 484 / 492; BF16 0.5M 9.7 / 13.0, 1.0M 18.7 / 20.3,
+// 2.0M 38.7 / 38.2, 20M 343 / 311.  AA from 750k sites: at large FP32 lattices it
+// gives up 2-3 % for half of the population memory.
 constexpr int64_t AA_MIN_SITES = 750000;
 int32_t resolve_scheme(int32_t scheme, int64_t n) {
   if (scheme != HLB_SCHEME_AUTO) return scheme;
