@@ -699,13 +699,19 @@ extern "C" int hlb_step(hlb_solver* h, int64_t nsteps) {
   for (int64_t s = 0; s < nsteps; ++s) {
     if (h->scheme == HLB_PULL_AB && h->phase == HLB_READ_GATHER_AB) {
       if (const int m = hlb_multi_steps(h, nsteps - s)) {
-        CUDA_TRY(hlb_launch_multi(h, h->f[h->cur], h->f[h->cur ^ 1], h->t, m, h->stream));
-        h->cur ^= 1;
-        h->t += m;
-        h->stepped = true;
-        if (h->any_wk()) CUDA_TRY(hlb_launch_wk_update(h, h->f[h->cur], h->t - 1, true, h->stream));
-        s += m - 1;
-        continue;
+        const cudaError_t e = hlb_launch_multi(h, h->f[h->cur], h->f[h->cur ^ 1], h->t, m, h->stream);
+        if (e == cudaSuccess) {
+          h->cur ^= 1;
+          h->t += m;
+          h->stepped = true;
+          if (h->any_wk()) CUDA_TRY(hlb_launch_wk_update(h, h->f[h->cur], h->t - 1, true, h->stream));
+          s += m - 1;
+          continue;
+        }
+        // fewer SMs than the device has (a partitioned GPU): launch by launch from here on
+        if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return hlb_cuda_fail(e, "hlb_step");
+        cudaGetLastError();
+        h->multi_blocks = 0;
       }
     }
     if (h->scheme == HLB_AA) {

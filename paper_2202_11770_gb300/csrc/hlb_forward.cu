@@ -1227,6 +1227,16 @@ cudaError_t dispatch(int precision, A... a) {
 inline unsigned iolet_blocks(const hlb_solver* h, int threads) {
   return (unsigned)((h->n_iolet_sites * kStepIoletLanes + threads - 1) / threads);
 }
+// Prefetch distance of the two-site kernels, in tiles.  An FP32 state that stays
+// in L2 has nothing to fetch ahead, and the hints for its rows only cost: none
+// below 600k sites.
+template <typename S>
+uint32_t pair_prefetch(const hlb_solver* h) {
+  return sizeof(S) == 4 && h->n < 600000 ? 0u : (uint32_t)h->n_sm * 3u;
+}
+// 16-bit AA odd steps of fewer sites take one site a thread: a wave of the chip
+// holds them all, and the shorter thread is done sooner.
+constexpr int64_t kOddPairSites = 200000;
 constexpr int64_t kSpreadSites = 4000000;
 inline uint32_t spread_factor(uint32_t iolet, uint32_t blocks) {
   return blocks ? (uint32_t)((((uint64_t)iolet << 32) + blocks - 1) / blocks) : 0u;
@@ -1266,7 +1276,7 @@ cudaError_t launch_gather(const hlb_solver* h, const void* fin, void* fout, cons
   // a whole step past L2: the iolet blocks beside their sites (FP32 8.0M sites 215 -> 204 us, 20M 497 -> 483;
   // 16 bits the same); a small lattice, or a part of the step: evenly among its tiles, which needs no search
   // (0.5M sites, BF16: 10.0 us a step, 10.5 with it)
-  const bool whole = iolets && tile0 == 0 && ntiles == grid_for(h->n) && h->n >= kSpreadSites;
+  const bool whole = iolets && tile0 == 0 && ntiles == grid_for(h->n) && (h->n >= kSpreadSites || sizeof(S) == 8);
   IoletSpread spread;
   if (ntiles == 0) tile0 = kNoTile;
   if constexpr (sizeof(S) <= 4) {
@@ -1275,7 +1285,7 @@ cudaError_t launch_gather(const hlb_solver* h, const void* fin, void* fout, cons
                                   : spread_evenly(ntiles, iolets ? iolet_blocks(h, PAIR) : 0u, &spread);
       if (grid == 0) return cudaSuccess;
       return launch_pdl(h->off32 ? k_step2<S, false> : k_step2<S, true>, grid, PAIR, s, (const S*)fin, (S*)fout, h->index(),
-                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, spread, (uint32_t)h->n_sm * 3u, tile0, p);
+                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, spread, pair_prefetch<S>(h), tile0, p);
     }
   }
   const unsigned grid = whole ? spread_iolets(h, BLOCK, BLOCK, &spread)
@@ -1331,14 +1341,14 @@ cudaError_t launch_aa(const hlb_solver* h, S* A, bool odd, const StepParams& p, 
   const unsigned g = grid_for(h->n);
   if (odd) {
     if constexpr (sizeof(S) <= 4) {
-      if (h->compact) {
+      if (h->compact && (sizeof(S) == 4 || h->n >= kOddPairSites)) {
         const AAIolets io = aa_iolets<GRID>(h, g, PAIR);
         return launch_pdl(h->off32 ? k_aa_odd2<S, false, GRID> : k_aa_odd2<S, true, GRID>, g + io.blocks, PAIR, s, A,
-                          h->index(), io, (uint32_t)h->n_sm * 3u, p);
+                          h->index(), io, pair_prefetch<S>(h), p);
       }
     }
     if constexpr (!GRID) {
-      constexpr bool CT = sizeof(S) > 4;  // FP64 only: the others take two sites a thread
+      constexpr bool CT = sizeof(S) != 4;  // FP32 takes two sites a thread
       return launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, CT> : k_aa_odd<S, true, CT>)
                                    : (h->off32 ? k_aa_odd<S, false, false> : k_aa_odd<S, true, false>),
                         g, BLOCK, s, A, h->index(), (uint32_t)h->n_sm * (h->off32 ? 3u : 4u), p);
