@@ -58,7 +58,8 @@ enum hlb_status {
   HLB_ERR_CUDA = -3,     /* a CUDA runtime call failed                        */
   HLB_ERR_STATE = -4,    /* call not valid in the solver's current state      */
   HLB_ERR_DIVERGED = -5, /* non-finite mass: the run has blown up             */
-  HLB_ERR_NOMEM = -6     /* host allocation failed                            */
+  HLB_ERR_NOMEM = -6,    /* host allocation failed                            */
+  HLB_ERR_WAIT = -7      /* a wait inside a multi-step launch ran out         */
 };
 enum hlb_precision { HLB_FP32 = 0, HLB_BF16 = 1, HLB_FP16 = 2, HLB_FP64 = 3 };
 enum hlb_scheme { HLB_SCHEME_AUTO = 0, HLB_PULL_AB = 1, HLB_AA = 2 };
@@ -229,7 +230,10 @@ int hlb_init_equilibrium(hlb_solver* h, double rho0, const float* u0, int32_t wh
  * scheme on a large lattice, a boundary pass over the iolet sites, plus one
  * small update kernel when Windkessel outlets are set.  A small lattice of the
  * pull scheme takes all n steps (n >= 4) in one launch, or a few, outside a
- * stream capture. */
+ * stream capture.  Its blocks pass populations to one another with waits that
+ * are bounded: should one run out, the state is no longer valid, and every
+ * synchronising call returns HLB_ERR_WAIT until hlb_init_equilibrium or
+ * hlb_set_state sets a new one (device outputs hold NaN). */
 int hlb_step(hlb_solver* h, int64_t n);
 int hlb_time(const hlb_solver* h, int64_t* t);
 

@@ -766,6 +766,7 @@ int run_adjoint(hlb_solver* h, int64_t N, const hlb_objective* obj, char* ws, co
   if (dtau_out) *dtau_out = host[1];
   if (damp)
     for (int k = 0; k < G; ++k) damp[k] = host[2 + k];
+  if (const int rc = hlb_check_waits(h)) return rc;
   if (!std::isfinite(host[0]) || !std::isfinite(host[1])) return hlb_fail(HLB_ERR_DIVERGED, "non-finite adjoint");
   return HLB_OK;
 }

@@ -392,6 +392,7 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   h->d_stage = (float*)(base + y.stage);
   h->d_red = (double*)(base + y.red);
   h->red_slots = hlb_reduce_slots(n, h->n_iolets);
+  h->d_status = (uint32_t*)(h->d_red + h->red_slots - 1);
   h->d_lflux = (double*)(base + y.lflux);
   h->d_iolet_sites = (int32_t*)(base + y.isites);
   h->d_icode = (int32_t*)(base + y.icode);
@@ -546,7 +547,8 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
     e = cudaMemcpyAsync(h->d_ioff, ioff.data(), sizeof(int64_t) * ioff.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !ilist.empty())
     e = cudaMemcpyAsync(h->d_ilist, ilist.data(), sizeof(int32_t) * ilist.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && h->multi_blocks > 0)
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->d_status, 0, sizeof(double), st);
+  if (e == cudaSuccess && h->d_word)
     e = cudaMemsetAsync(h->d_word, 0, sizeof(uint64_t) * hlb_multi_words(n, y.n_links, h->n_iolets, h->precision), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_lflux, 0, sizeof(double) * (size_t)std::max<int64_t>(y.n_links, 1), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->f[0], 0, h->state_bytes(), st);  // rest: h = f - w = 0
@@ -668,6 +670,7 @@ extern "C" int hlb_windkessel_state(hlb_solver* h, int32_t k, double* rho_ghost,
   const double* g = h->scheme == HLB_AA ? h->d_ioval : h->d_iovnext;
   CUDA_TRY(cudaMemcpyAsync(&val, g + k, sizeof val, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
+  if (const int rc = hlb_check_waits(h)) return rc;
   if (rho_ghost) *rho_ghost = 1.0 + val;
   if (rho_c) *rho_c = state[0];
   if (q) *q = state[1];
@@ -682,6 +685,7 @@ extern "C" int hlb_init_equilibrium(hlb_solver* h, double rho0, const float* u0,
     CUDA_TRY(cudaMemcpyAsync(h->d_stage, u0, sizeof(float) * 3 * (size_t)h->n, cudaMemcpyHostToDevice, h->stream));
     du = h->d_stage;
   }
+  CUDA_TRY(hlb_clear_waits(h));
   CUDA_TRY(hlb_launch_init(h, h->f[0], rho0, du, h->stream));
   if (h->any_wk()) CUDA_TRY(hlb_launch_wk_reset(h, h->stream));
   h->cur = 0;
@@ -755,7 +759,7 @@ extern "C" int hlb_read_macros(hlb_solver* h, float* rho, float* u, float* wss, 
   if (u) CUDA_TRY(cudaMemcpyAsync(u, su, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, h->stream));
   if (wss) CUDA_TRY(cudaMemcpyAsync(wss, sw, sizeof(float) * n, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
-  return HLB_OK;
+  return hlb_check_waits(h);
 }
 
 // Mass, fluxes and (monitor) per-iolet max |u| and mean rho of the current
@@ -764,7 +768,7 @@ static int sums_impl(hlb_solver* h, double* mass, double* flux, bool monitor, do
   const int K = h->n_iolets;
   double* out = h->d_red + hlb_reduce_partials(h->n) + (K + 1);
   CUDA_TRY(hlb_launch_reduce(h, h->f[h->cur], h->phase, h->t - 1, h->stepped, monitor, out, h->stream));
-  std::vector<double> host((size_t)(monitor ? 1 + 3 * K : 1 + K));
+  std::vector<double> host((size_t)(1 + 3 * K + 1));  // the monitor's slots without it: left alone
   CUDA_TRY(cudaMemcpyAsync(host.data(), out, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
   if (mass) *mass = host[0];
@@ -773,6 +777,9 @@ static int sums_impl(hlb_solver* h, double* mass, double* flux, bool monitor, do
     if (u_max) u_max[k] = host[(size_t)(1 + K + k)];
     if (rho_mean) rho_mean[k] = host[(size_t)(1 + 2 * K + k)];
   }
+  uint32_t late;
+  memcpy(&late, &host[(size_t)(1 + 3 * K)], sizeof late);
+  if (const int rc = hlb_wait_status(h, late)) return rc;
   if (!std::isfinite(host[0])) return hlb_fail(HLB_ERR_DIVERGED, "mass is not finite");
   return HLB_OK;
 }
@@ -827,13 +834,17 @@ extern "C" int hlb_get_state(hlb_solver* h, void* f, int32_t where, int64_t* t) 
     }
   }
   if (t) *t = h->t;
-  if (where == HLB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream));
+  if (where == HLB_HOST) {
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    return hlb_check_waits(h);
+  }
   return HLB_OK;
 }
 
 extern "C" int hlb_set_state(hlb_solver* h, const void* f, int32_t where, int64_t t) {
   if (!h || !f) return hlb_fail(HLB_ERR_ARG, "null argument");
   if (t < 0) return hlb_fail(HLB_ERR_ARG, "negative time");
+  CUDA_TRY(hlb_clear_waits(h));
   CUDA_TRY(cudaMemcpyAsync(h->f[0], f, h->state_bytes(),
                            where == HLB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, h->stream));
   if (where == HLB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream));

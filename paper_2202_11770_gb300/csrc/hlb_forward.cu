@@ -1546,8 +1546,8 @@ int64_t hlb_reduce_partials(int64_t n) { return mass_blocks(n, mass_sites(n)); }
 
 int64_t hlb_reduce_slots(int64_t n, int32_t n_iolets) {
   // per-block partials, iolet link ranges (int64, n_iolets + 1), final outputs: mass and
-  // fluxes (1 + n_iolets), monitor (2 n_iolets)
-  return hlb_reduce_partials(n) + (n_iolets + 1) + (1 + 3 * (int64_t)n_iolets);
+  // fluxes (1 + n_iolets), monitor (2 n_iolets), then the status word of the multi-step launches
+  return hlb_reduce_partials(n) + (n_iolets + 1) + (1 + 3 * (int64_t)n_iolets) + 1;
 }
 
 cudaError_t hlb_launch_step(const hlb_solver* h, const void* fin, void* fout, bool gather, int64_t tb,

@@ -16,6 +16,13 @@
 // How read-back kernels obtain f(t) from a population buffer.
 enum { HLB_READ_LOCAL = 0, HLB_READ_GATHER_AB = 1, HLB_READ_GATHER_AA = 2 };
 
+// The waits of a multi-step launch (hlb_multi.cu): a bulk site's and an iolet
+// site's for the populations they gather, a link's for its outlet's ghost
+// density, an outlet's for its link masses.
+namespace hlb {
+enum { WAIT_BULK = 0, WAIT_IOLET, WAIT_GHOST, WAIT_FLUX, kMultiWaits };
+}
+
 struct HostWave {
   int32_t kind = HLB_WAVE_CONST;
   double mean = 0, rel = 0, period = 1, phase = 0;
@@ -91,6 +98,9 @@ struct hlb_solver {
   uint64_t* d_word = nullptr;         // words that pass between sites (hlb_multi_words)
   int multi_blocks = 0;               // blocks that fit on the device at once, 0: steps are launched one by one
   uint32_t multi_tag = 1;             // number of the next such step (0: never written)
+  uint32_t multi_limit[hlb::kMultiWaits] = {1u << 22, 1u << 22, 1u << 22, 1u << 22};  // polls (half a microsecond or more each) of a wait
+  uint32_t* d_status = nullptr;       // set by a wait that ran out (after the outputs of d_red)
+  bool multi_ran = false;             // such a launch since the state was last set: d_status may be set
   bool any_wk() const {
     for (int v : wk_on)
       if (v) return true;
@@ -156,6 +166,16 @@ size_t hlb_multi_words(int64_t n, int64_t n_links, int32_t n_iolets, int32_t pre
 int hlb_multi_blocks(const hlb_solver* h);
 // Steps that the next launch may take towards `left` more, 0: launch them one by one.
 int hlb_multi_steps(const hlb_solver* h, int64_t left);
+// HLB_ERR_WAIT when a wait of a launch since the state was last set ran out
+// (one small copy and a synchronisation, when there was such a launch at all).
+int hlb_check_waits(hlb_solver* h);
+// The same from the status word that a caller has already copied back.
+int hlb_wait_status(hlb_solver* h, uint32_t late);
+// The state is about to be set anew: forget such a wait.
+cudaError_t hlb_clear_waits(hlb_solver* h);
+// For tests: the poll limit of each kind of wait, the number of the next step
+// (0: leave it) and the number of blocks taken to fit on the device (0: leave it).
+extern "C" int hlb_multi_test(hlb_solver* h, const uint32_t* limits, uint32_t next_step, int blocks);
 // m pull A-B gather steps from `in`, which holds s'(t - 1); the last is stored to `out`.
 cudaError_t hlb_launch_multi(hlb_solver* h, const void* in, void* out, int64_t t, int m, cudaStream_t s);
 

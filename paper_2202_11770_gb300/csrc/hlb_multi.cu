@@ -23,8 +23,10 @@
 // hands the next ghost density back, both through words of the same kind.
 //
 // Every wait is bounded.  The cooperative launch makes all blocks resident, so
-// no wait runs out in a correct run; a thread whose wait does leaves NaN in
-// its populations, which the mass reduction reports as a run that has blown up.
+// no wait runs out in a correct run.  A thread whose wait does run out sets the
+// solver's status word, which the next synchronising call returns as
+// HLB_ERR_WAIT, leaves NaN in what it would have written (its site's
+// populations, its outlet's model) and returns.
 #include <algorithm>
 
 #include "hlb_internal.h"
@@ -34,7 +36,6 @@ using namespace hlb;
 namespace {
 
 constexpr int TB = 64;                     // threads a block
-constexpr unsigned kSpinLimit = 1u << 22;  // polls of half a microsecond or more
 // A thread whose words have not all come sleeps this long before it asks again:
 // the polls of the others load L2 less (50k sites 4.1 -> 3.8 us a step).
 constexpr unsigned kPollSleep = 100;  // ns
@@ -55,6 +56,8 @@ struct MultiArgs {
   uint64_t* flux;         // [links][2] link masses, FP64 words
   uint64_t* ghost;        // [iolets][2] ghost densities less 1, FP64 words
   uint32_t tag0;          // number of the launch's first step
+  uint32_t limit[kMultiWaits];  // polls after which a wait of each kind (WAIT_BULK ..) gives up
+  uint32_t* status;       // set to 1 by a wait that ran out
   int32_t nbulk, niolet, nsteps;
   // Windkessel outlets
   const int64_t* begin;   // link ranges per iolet
@@ -99,11 +102,11 @@ template <> struct Word<double> {
   }
 };
 // One value, waited for; *late set when the wait runs out.
-__device__ __forceinline__ double wait_double(const uint64_t* p, uint32_t tag, bool* late) {
+__device__ __forceinline__ double wait_double(const uint64_t* p, uint32_t tag, uint32_t limit, bool* late) {
   Word<double> v;
   unsigned spins = 0;
   for (v.load(p); !v.is(tag); v.load(p))
-    if (++spins > kSpinLimit) {
+    if (++spins > limit) {
       *late = true;
       break;
     }
@@ -118,6 +121,7 @@ template <typename S>
 __device__ __forceinline__ S not_a_number() {
   return from_real<S>(typename Real<S>::type(__int_as_float(0x7fc00000)));
 }
+__device__ __forceinline__ void ran_out(const MultiArgs& a) { *(volatile uint32_t*)a.status = 1u; }
 
 template <typename S>
 __device__ __forceinline__ void bulk_block(const S* in, S* out, const MultiArgs& a, const StepParams& p, int b) {
@@ -156,8 +160,10 @@ __device__ __forceinline__ void bulk_block(const S* in, S* out, const MultiArgs&
       for (int i = 1; i < Q; ++i) all &= w[i].is(tag);
       if (all) break;
       if (sizeof(S) < 8) __nanosleep(kPollSleep);  // FP64: 11.6 us a step without, 17.7 with
-      if (++spins > kSpinLimit) {
-        out[x] = not_a_number<S>();
+      if (++spins > a.limit[WAIT_BULK]) {
+#pragma unroll 1
+        for (int i = 0; i < Q; ++i) out[(uint32_t)i * n + x] = not_a_number<S>();
+        ran_out(a);
         return;
       }
     }
@@ -197,6 +203,14 @@ __device__ __forceinline__ void iolet_block(const S* in, S* out, const MultiArgs
     own[e] = i < Q ? to_real(in[(uint32_t)i * n + x]) : R(0);
   }
   const R omega = omega_of<R>(p);
+  // A wait of some lane of the warp ran out: the warp's sites end here.
+  auto give_up = [&](bool late) {
+    if (!__any_sync(FULL_MASK, late)) return false;
+#pragma unroll 1
+    for (int i = hl; live && i < Q; i += W) out[(uint32_t)i * n + x] = not_a_number<S>();
+    if (late) ran_out(a);
+    return true;
+  };
   for (int k = 0;; ++k) {
     const bool last = k == a.nsteps - 1;
     uint64_t* put = a.word + (int64_t)(k & 1) * (Q - 1) * n * WD::N;
@@ -220,7 +234,7 @@ __device__ __forceinline__ void iolet_block(const S* in, S* out, const MultiArgs
         R val = wave.v[k * K + io[e]];
         const bool coupled = (p.coupled[io[e] >> 6] >> (io[e] & 63)) & 1ull;
         // the outlet's block sends the ghost density of step k >= 2 with that step's number
-        if (coupled && live) val = R(k == 0 ? p.ioval[io[e]] : (k == 1 ? a.iovnext[io[e]] : wait_double(a.ghost + 2 * io[e], tag, &late)));
+        if (coupled && live) val = R(k == 0 ? p.ioval[io[e]] : (k == 1 ? a.iovnext[io[e]] : wait_double(a.ghost + 2 * io[e], tag, a.limit[WAIT_GHOST], &late)));
         const R o = h[e];
         LinkRec L;
         L.kind = (int8_t)kind[e];
@@ -235,6 +249,7 @@ __device__ __forceinline__ void iolet_block(const S* in, S* out, const MultiArgs
           Word<double>::store(a.flux + 2 * (int64_t)(-c[e] - 2), (double)m - (double)o, tag);
         }
       }
+    if (give_up(late)) return;
     R drho = __shfl_sync(FULL_MASK, h[0], 0, W), cjx = R(0), cjy = R(0), cjz = R(0);
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
@@ -271,15 +286,12 @@ __device__ __forceinline__ void iolet_block(const S* in, S* out, const MultiArgs
         }
       }
       if (all) break;
-      if (++spins > kSpinLimit) {
+      if (++spins > a.limit[WAIT_IOLET]) {
         late = true;
         break;
       }
     }
-    if (__any_sync(FULL_MASK, late)) {
-      if (live && hl == 0) out[x] = not_a_number<S>();
-      return;
-    }
+    if (give_up(late)) return;
 #pragma unroll
     for (int e = 0; e < NE; ++e) {
       const int i = e * W + hl;
@@ -319,13 +331,17 @@ __device__ __forceinline__ void wk_block(const MultiArgs& a, const StepParams& p
         for (int u = 0; u < 8; ++u)
           if (r + u * TB < hi) all &= v[u].is(tag);
         if (all) break;
-        late = ++spins > kSpinLimit;
+        late = ++spins > a.limit[WAIT_FLUX];
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (r + u * TB < hi) acc += v[u].value();
     }
-    if (__syncthreads_or(late)) return;
+    if (__syncthreads_or(late)) {
+      if (late) ran_out(a);
+      if (threadIdx.x == 0) a.wkstate[2 * io] = a.wkstate[2 * io + 1] = a.iovnext[io] = __longlong_as_double(0x7ff8000000000000ll);
+      return;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(FULL_MASK, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -407,6 +423,8 @@ cudaError_t launch(hlb_solver* h, const void* in, void* out, int64_t t, int m, c
   a.flux = h->d_word + 2 * (Q - 1) * h->n * Word<R>::N;
   a.ghost = a.flux + 2 * h->n_links;
   a.tag0 = h->multi_tag;
+  for (int k = 0; k < kMultiWaits; ++k) a.limit[k] = h->multi_limit[k];
+  a.status = h->d_status;
   a.nbulk = bulk_blocks(h->n);
   a.niolet = iolet_blocks(h->n_iolet_sites);
   a.nsteps = m;
@@ -426,7 +444,10 @@ cudaError_t launch(hlb_solver* h, const void* in, void* out, int64_t t, int m, c
   const cudaError_t e = cudaLaunchKernelEx(&cfg, k_multi<S>, (const S*)in, (S*)out, (const MultiArgs)a,
                                            (const WaveTable<R>)wave, p);
   // step numbers are never used twice, so no word of an earlier launch is taken for a new one
-  if (e == cudaSuccess) h->multi_tag += (uint32_t)m;
+  if (e == cudaSuccess) {
+    h->multi_tag += (uint32_t)m;
+    h->multi_ran = true;
+  }
   return e;
 }
 
@@ -471,6 +492,35 @@ int hlb_multi_steps(const hlb_solver* h, int64_t left) {
   }
   const int64_t most = h->n_iolets > 0 ? kMultiVals / h->n_iolets : kMultiVals;
   return (int)std::min(left, most);
+}
+
+int hlb_check_waits(hlb_solver* h) {
+  if (!h->multi_ran) return HLB_OK;
+  uint32_t late = 0;
+  cudaError_t e = cudaMemcpyAsync(&late, h->d_status, sizeof late, cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e != cudaSuccess) return hlb_cuda_fail(e, "status of a multi-step launch");
+  return hlb_wait_status(h, late);
+}
+
+int hlb_wait_status(hlb_solver* h, uint32_t late) {
+  if (late) return hlb_fail(HLB_ERR_WAIT, "a wait inside a multi-step launch ran out: the state is not valid");
+  h->multi_ran = false;
+  return HLB_OK;
+}
+
+cudaError_t hlb_clear_waits(hlb_solver* h) {
+  if (!h->multi_ran) return cudaSuccess;
+  h->multi_ran = false;
+  return cudaMemsetAsync(h->d_status, 0, sizeof(double), h->stream);
+}
+
+extern "C" int hlb_multi_test(hlb_solver* h, const uint32_t* limits, uint32_t next_step, int blocks) {
+  if (!h || !limits) return hlb_fail(HLB_ERR_ARG, "null argument");
+  for (int k = 0; k < kMultiWaits; ++k) h->multi_limit[k] = limits[k];
+  if (next_step) h->multi_tag = next_step;
+  if (blocks && h->d_word) h->multi_blocks = blocks;
+  return HLB_OK;
 }
 
 cudaError_t hlb_launch_multi(hlb_solver* h, const void* in, void* out, int64_t t, int m, cudaStream_t s) {

@@ -22,6 +22,7 @@ import numpy as np
 _LIB_PATH = Path(__file__).resolve().parent / "_lib" / "libhemegb.so"
 
 HLB_OK, HLB_ERR_ARG, HLB_ERR_WS, HLB_ERR_CUDA, HLB_ERR_STATE, HLB_ERR_DIVERGED, HLB_ERR_NOMEM = 0, -1, -2, -3, -4, -5, -6
+HLB_ERR_WAIT = -7
 HLB_FP32, HLB_BF16, HLB_FP16, HLB_FP64 = 0, 1, 2, 3
 HLB_SCHEME_AUTO, HLB_PULL_AB, HLB_AA = 0, 1, 2
 HLB_VELOCITY, HLB_PRESSURE = 0, 1
