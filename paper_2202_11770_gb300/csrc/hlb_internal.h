@@ -16,11 +16,11 @@
 // How read-back kernels obtain f(t) from a population buffer.
 enum { HLB_READ_LOCAL = 0, HLB_READ_GATHER_AB = 1, HLB_READ_GATHER_AA = 2 };
 
-// The waits of a multi-step launch (hlb_multi.cu): a bulk site's and an iolet
-// site's for the populations they gather, a link's for its outlet's ghost
-// density, an outlet's for its link masses.
+// The waits of a multi-step launch (hlb_multi.cu) whose limits are arguments: a
+// bulk site's and an iolet site's for the populations they gather, an outlet's
+// for its link masses.
 namespace hlb {
-enum { WAIT_BULK = 0, WAIT_IOLET, WAIT_GHOST, WAIT_FLUX, kMultiWaits };
+enum { WAIT_BULK = 0, WAIT_IOLET, WAIT_FLUX, kMultiWaits };
 }
 
 struct HostWave {
@@ -98,7 +98,7 @@ struct hlb_solver {
   uint64_t* d_word = nullptr;         // words that pass between sites (hlb_multi_words)
   int multi_blocks = 0;               // blocks that fit on the device at once, 0: steps are launched one by one
   uint32_t multi_tag = 1;             // number of the next such step (0: never written)
-  uint32_t multi_limit[hlb::kMultiWaits] = {1u << 22, 1u << 22, 1u << 22, 1u << 22};  // polls (half a microsecond or more each) of a wait
+  uint32_t multi_limit[hlb::kMultiWaits] = {1u << 22, 1u << 22, 1u << 22};  // polls (half a microsecond or more each) of a wait
   uint32_t* d_status = nullptr;       // set by a wait that ran out (after the outputs of d_red)
   bool multi_ran = false;             // such a launch since the state was last set: d_status may be set
   bool any_wk() const {

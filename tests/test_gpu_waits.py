@@ -19,15 +19,15 @@ pytestmark = pytest.mark.gpu
 hemegb = pytest.importorskip("paper_2202_11770_gb300.hemegb")
 torch = pytest.importorskip("torch")
 
-KINDS = ["bulk", "iolet", "ghost", "flux"]
+KINDS = ["bulk", "iolet", "flux"]
 POLLS = 1 << 22
 
 
-def _tune(s, limits=(POLLS,) * 4, next_step=0, blocks=0):
+def _tune(s, limits=(POLLS,) * len(KINDS), next_step=0, blocks=0):
     """hlb_multi_test: poll limits by kind, number of the next step, blocks taken to fit."""
     fn = hemegb.library().hlb_multi_test
     fn.argtypes = [C.c_void_p, C.POINTER(C.c_uint32), C.c_uint32, C.c_int]
-    assert fn(s.handle, (C.c_uint32 * 4)(*limits), next_step, blocks) == hemegb.HLB_OK
+    assert fn(s.handle, (C.c_uint32 * len(KINDS))(*limits), next_step, blocks) == hemegb.HLB_OK
 
 
 def _start(lat, prec="fp32", windkessel=True):
@@ -60,7 +60,9 @@ def test_a_wait_that_runs_out_is_reported(kind, steps):
     s = _start(lat)
     s.step(9)
     s.reduce()                                   # a sound launch reports nothing
-    _tune(s, [0 if k == kind else 1 << 14 for k in KINDS])
+    # without its link masses an outlet's block gives up, and its links' wait for the ghost density
+    # runs out by itself before the others do
+    _tune(s, [0 if k == kind else POLLS if kind == "flux" else 1 << 14 for k in KINDS])
     s.step(steps)
     for call in (s.reduce, s.state, s.macros, s.iolet_monitor, lambda: s.windkessel_state(1), s.reduce):
         assert _code(call) == hemegb.HLB_ERR_WAIT
