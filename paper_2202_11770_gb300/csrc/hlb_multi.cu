@@ -409,6 +409,13 @@ int resident_blocks(int n_sm) {
 template <typename S>
 cudaError_t launch(hlb_solver* h, const void* in, void* out, int64_t t, int m, cudaStream_t s) {
   using R = typename Real<S>::type;
+  if (h->multi_tag > UINT32_MAX - (uint32_t)m) {
+    // the step numbers start again: clear the words first, so that none left from 2^32
+    // steps ago, or never written, is taken for a new one
+    const cudaError_t e = cudaMemsetAsync(h->d_word, 0, sizeof(uint64_t) * hlb_multi_words(h->n, h->n_links, h->n_iolets, h->precision), s);
+    if (e != cudaSuccess) return e;
+    h->multi_tag = 1;
+  }
   const StepParams p = h->params(t);
   WaveTable<R> wave;
   const int K = h->n_iolets;
@@ -447,7 +454,8 @@ cudaError_t launch(hlb_solver* h, const void* in, void* out, int64_t t, int m, c
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, k_multi<S>, (const S*)in, (S*)out, (const MultiArgs)a,
                                            (const WaveTable<R>)wave, p);
-  // step numbers are never used twice, so no word of an earlier launch is taken for a new one
+  // no step number is used twice without the words being cleared in between, so no word of an
+  // earlier launch is taken for a new one
   if (e == cudaSuccess) {
     h->multi_tag += (uint32_t)m;
     h->multi_ran = true;

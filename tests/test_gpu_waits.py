@@ -118,3 +118,20 @@ def test_solvers_on_two_streams():
         for s in runs:
             s.step(200)
     assert [s.state()[0].tobytes() for s in runs] == want
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("before", [1, 2, 37, 38])
+def test_step_numbers_that_start_again(before, prec):
+    """The 32-bit step numbers run out `before` steps into a run of 37 with
+    outlet models: the numbers after that must not match the words that hold
+    no number yet (0)."""
+    lat = geo.pipe(8.0, 64)
+    a, b = _start(lat, prec), _start(lat, prec)
+    _tune(a, next_step=2 ** 32 - before)
+    for s in (a, b):
+        s.step(1)
+        s.step(37)
+        s.step(20)
+    assert a.state()[0].tobytes() == b.state()[0].tobytes()
+    assert a.windkessel_state(1) == b.windkessel_state(1)
