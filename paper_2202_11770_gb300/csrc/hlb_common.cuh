@@ -782,6 +782,17 @@ __device__ __forceinline__ double site_sum(const float* h) {
   for (int i = 0; i < Q; ++i) d += (double)h[i];
   return d;
 }
+// The Windkessel model of an outlet one step on, q its outflow in that step:
+// advances rho_c and returns the next ghost density less 1.
+__device__ __forceinline__ double wk_advance(double Rp, double C, double Rd, double rho_d, double q, double* rho_c) {
+  if (!(C > 0)) return fmadd(Rp + Rd, q, rho_d) - 1.0;
+  *rho_c += (q - (*rho_c - rho_d) / Rd) / C;
+  return fmadd(Rp, q, *rho_c) - 1.0;
+}
+// An outlet's link masses are summed by this many lanes, lane l its links l,
+// l + kWkLanes, .. in order, then the lanes of a warp, then the warps.
+constexpr int kWkLanes = 64;
+
 // Sites a thread of a mass reduction over a lattice of n takes (a block: that
 // many x 256): four, so that the FP64 block sum is paid once for them, but one
 // below a million sites, where four sites in a chain take longer than they

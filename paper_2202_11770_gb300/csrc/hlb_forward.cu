@@ -1417,7 +1417,7 @@ __global__ void __launch_bounds__(BLOCK) k_wk_update(const S* __restrict__ fin, 
                                                      const double* __restrict__ par, double* __restrict__ state,
                                                      double* ioval, double* __restrict__ iovnext, int shift) {
   using R = typename Real<S>::type;
-  __shared__ double sh[BLOCK / 32];
+  __shared__ double sh[BLOCK / 32], mass[BLOCK];
   const int k = blockIdx.x;
   pdl_wait();
   pdl_trigger();
@@ -1428,9 +1428,12 @@ __global__ void __launch_bounds__(BLOCK) k_wk_update(const S* __restrict__ fin, 
   }
   const int64_t n = p.n;
   double acc = 0;
-  for (int64_t r = begin[k] + threadIdx.x; r < begin[k + 1]; r += BLOCK) {
-    if (AA) {
-      acc += lflux[r];
+  for (int64_t r0 = begin[k], end = begin[k + 1]; r0 < end; r0 += BLOCK) {
+    const int64_t r = r0 + threadIdx.x;
+    if (r >= end) {
+      mass[threadIdx.x] = 0;
+    } else if (AA) {
+      mass[threadIdx.x] = lflux[r];
     } else {
       const LinkRec L = links[r];
       const int64_t x = L.site;
@@ -1446,23 +1449,24 @@ __global__ void __launch_bounds__(BLOCK) k_wk_update(const S* __restrict__ fin, 
 #pragma unroll
       for (int i = 1; i < Q; ++i)
         if (i == j) val = iolet_value<R>(i, L, out, ms.rho, ms.ux, ms.uy, ms.uz, amp, p);
-      acc += (double)val - (double)out;
+      mass[threadIdx.x] = (double)val - (double)out;
     }
+    // in the order of a multi-step launch's outlet blocks (hlb_multi.cu); the zeros past the end add nothing
+    __syncthreads();
+    if (threadIdx.x < kWkLanes) {
+#pragma unroll
+      for (int u = 0; u < BLOCK / kWkLanes; ++u) acc += mass[threadIdx.x + u * kWkLanes];
+    }
+    __syncthreads();
   }
   const double flux = block_sum(acc, sh);
   if (threadIdx.x == 0) {
     const double Rp = par[4 * k], C = par[4 * k + 1], Rd = par[4 * k + 2], rho_d = par[4 * k + 3];
     const double q = -flux;
-    double rho_c = state[2 * k], ghost;
-    if (C > 0) {
-      rho_c += (q - (rho_c - rho_d) / Rd) / C;
-      ghost = rho_c + Rp * q;
-    } else {
-      ghost = rho_d + (Rp + Rd) * q;
-    }
+    double rho_c = state[2 * k];
+    (AA ? ioval : iovnext)[k] = wk_advance(Rp, C, Rd, rho_d, q, &rho_c);
     state[2 * k] = rho_c;
     state[2 * k + 1] = q;
-    (AA ? ioval : iovnext)[k] = ghost - 1.0;
   }
 }
 

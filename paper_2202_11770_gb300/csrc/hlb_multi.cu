@@ -305,11 +305,13 @@ __device__ __forceinline__ void iolet_block(const S* in, S* out, const MultiArgs
 }
 
 // The model of Windkessel outlet number j among the coupled ones, as
-// k_wk_update (hlb_forward.cu) advances it.  The gather of step k >= 1 applies
+// k_wk_update (hlb_forward.cu) advances it, its link masses summed in the same
+// order, so that a run gives the same bits however it is cut into launches.  The gather of step k >= 1 applies
 // the boundary values of the state that step k - 1 produced, so its link
 // masses are that state's outflow; they set the ghost density of step k + 1.
 // (The outflow after the last step is k_wk_update's, after this launch.)
 __device__ __forceinline__ void wk_block(const MultiArgs& a, const StepParams& p, int j) {
+  static_assert(TB == kWkLanes, "the order of the sum");
   __shared__ double sh[TB / 32];
   const int K = p.n_iolets;
   int io = -1;
@@ -354,13 +356,7 @@ __device__ __forceinline__ void wk_block(const MultiArgs& a, const StepParams& p
       double flux = 0;
       for (int w = 0; w < TB / 32; ++w) flux += sh[w];
       const double q = -flux;
-      double ghost;
-      if (C > 0) {
-        rho_c += (q - (rho_c - rho_d) / Rd) / C;
-        ghost = rho_c + Rp * q - 1.0;
-      } else {
-        ghost = rho_d + (Rp + Rd) * q - 1.0;
-      }
+      const double ghost = wk_advance(Rp, C, Rd, rho_d, q, &rho_c);
       if (k == a.nsteps - 1) {
         a.wkstate[2 * io] = rho_c;
         a.wkstate[2 * io + 1] = q;
