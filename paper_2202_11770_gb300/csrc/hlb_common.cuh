@@ -752,36 +752,69 @@ __device__ __forceinline__ uint32_t load_state(const S* __restrict__ fin, const 
 }
 
 // ---------------------------------------------------------------------------
-// Sum of a site's 19 populations for the FP64 mass reductions.  GB300 runs
-// FP64 additions and conversions at 1/64 of the FP32 rate, and 38 of them a
-// site made the reduction take 2.8 times its memory time.  FP32 values are
-// therefore summed as an unevaluated pair hi + lo (Knuth's two-sum: the
-// rounding error of every addition is exact in FP32 and goes to lo), and the
-// pair is converted once.  lo is some 2^-24 of hi and carries a rounding error
-// of 2^-24 of itself, below what adding the site to a block's FP64 sum rounds
-// off.  A sum that leaves the FP32 range is taken again in FP64.
+// Sum of a thread's populations (19 of each of up to 4 sites) for the FP64 mass
+// reductions.  GB300 runs FP64 additions and conversions at 1/64 of the FP32
+// rate, and 38 of them a site made the reduction take 2.8 times its memory time.
+// FP32 values are therefore summed as an unevaluated triple hi + lo + lo2
+// (Knuth's two-sum: the rounding error of every addition is exact in FP32; those
+// of hi go to lo, those of lo to lo2), converted once a thread.  With u = 2^-24
+// and S the sum of the absolute values, only lo2 is rounded on the way: its m
+// terms (m <= 76) are u |lo| <= m u^2 S each, so at most m^3 u^3 S < 2^-53 S is
+// lost (one site: 2^-59 S), about one rounding of the m - 1 in a chain of FP64
+// additions.  (A pair hi + lo keeps only some 2^-43 of S.)  A sum that leaves
+// the FP32 range makes lo2 NaN: it is to be taken again in FP64.
+// FP32 snapshot of 8.0M sites (two steps, read-out, mass): 750 us; 753 with pairs,
+// 777 with a triple converted for every site.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double site_sum(const double* h) {
-  double d = 0;
-#pragma unroll
-  for (int i = 0; i < Q; ++i) d += h[i];
-  return d;
+// *a + b, rounded, into *a; returns the rounding error.
+__device__ __forceinline__ float two_sum(float* a, float b) {
+  const float s = __fadd_rn(*a, b), t = __fsub_rn(s, *a);
+  const float e = __fadd_rn(__fsub_rn(*a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  *a = s;
+  return e;
 }
-__device__ __forceinline__ double site_sum(const float* h) {
-  float hi = h[0], lo = 0.f;
+template <typename R> struct MassSum;
+template <> struct MassSum<double> {
+  double d = 0;
+  __device__ __forceinline__ void add(const double* h) {
 #pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const float s = __fadd_rn(hi, h[i]);
-    const float t = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(h[i], t)));
-    hi = s;
+    for (int i = 0; i < Q; ++i) d += h[i];
   }
-  if (isfinite(hi)) return (double)hi + (double)lo;
-  double d = 0;
+  __device__ __forceinline__ bool holds() const { return true; }
+  __device__ __forceinline__ double value() const { return d; }
+};
+template <> struct MassSum<float> {
+  float hi = 0.f, lo = 0.f, lo2 = 0.f;
+  __device__ __forceinline__ void add(const float* h) {
 #pragma unroll
-  for (int i = 0; i < Q; ++i) d += (double)h[i];
-  return d;
+    for (int i = 0; i < Q; ++i) lo2 = __fadd_rn(lo2, two_sum(&lo, two_sum(&hi, h[i])));
+  }
+  __device__ __forceinline__ bool holds() const { return isfinite(lo2); }
+  __device__ __forceinline__ double value() const { return (double)hi + ((double)lo + (double)lo2); }
+};
+// The sum over `count` sites, load(k, h) giving the k-th.
+template <typename R, typename Load>
+__device__ __forceinline__ double mass_sum(int count, Load&& load) {
+  MassSum<R> m;
+  double d = 0;
+#pragma unroll 1
+  for (bool wide = false;; wide = true) {
+#pragma unroll 1
+    for (int k = 0; k < count; ++k) {
+      R h[Q];
+      load(k, h);
+      if (wide) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) d += (double)h[i];
+      } else {
+        m.add(h);
+      }
+    }
+    if (wide) return d;
+    if (m.holds()) return m.value();
+  }
 }
+
 // The Windkessel model of an outlet one step on, q its outflow in that step:
 // advances rho_c and returns the next ghost density less 1.
 __device__ __forceinline__ double wk_advance(double Rp, double C, double Rd, double rho_d, double q, double* rho_c) {

@@ -1121,16 +1121,12 @@ __global__ void __launch_bounds__(BLOCK) k_sums(const S* __restrict__ fin, const
   const int64_t n = p.n;
   if (blockIdx.x < nmass) {
     __shared__ double sh[BLOCK / 32];
-    double d = 0;
     const int64_t x0 = lo + (int64_t)blockIdx.x * (per * BLOCK) + threadIdx.x;
-#pragma unroll 1
-    for (int k = 0; k < per; ++k) {
+    const int count = x0 >= hi ? 0 : (int)min((int64_t)per, (hi - x0 + BLOCK - 1) / BLOCK);
+    const double d = mass_sum<R>(count, [&](int k, R* h) {
       const int64_t x = x0 + k * BLOCK;
-      if (x >= hi) break;
-      R h[Q];
       load_state<S, MODE, CT, false>(fin, ix, links, amp, p, x, (uint32_t)(x / CT_TILE), h);
-      d += site_sum(h);
-    }
+    });
     const double s = block_sum(d, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
     return;

@@ -51,16 +51,11 @@ __global__ void __launch_bounds__(BLOCK) k_mass_static(const S* __restrict__ f, 
   using R = typename Real<S>::type;
   __shared__ double sh[BLOCK / 32];
   const int64_t x0 = (int64_t)blockIdx.x * (per * BLOCK) + threadIdx.x;
-  double d = 0;
-#pragma unroll 1
-  for (int k = 0; k < per; ++k) {
-    const int64_t x = x0 + k * BLOCK;
-    if (x >= n) break;
-    R h[Q];
+  const int count = x0 >= n ? 0 : (int)min((int64_t)per, (n - x0 + BLOCK - 1) / BLOCK);
+  const double d = mass_sum<R>(count, [&](int k, R* h) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) h[i] = ldpop(f + (int64_t)i * n + x);
-    d += site_sum(h);
-  }
+    for (int i = 0; i < Q; ++i) h[i] = ldpop(f + (int64_t)i * n + x0 + k * BLOCK);
+  });
   const double s = block_sum(d, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
