@@ -762,12 +762,12 @@ extern "C" int hlb_read_macros(hlb_solver* h, float* rho, float* u, float* wss, 
   return hlb_check_waits(h);
 }
 
-// Mass, fluxes and (monitor) per-iolet max |u| and mean rho of the current
-// state; one synchronisation.
-static int sums_impl(hlb_solver* h, double* mass, double* flux, bool monitor, double* u_max, double* rho_mean) {
+// (totals) mass and fluxes and (monitor) per-iolet max |u| and mean rho of the
+// current state; one synchronisation.
+static int sums_impl(hlb_solver* h, bool totals, double* mass, double* flux, bool monitor, double* u_max, double* rho_mean) {
   const int K = h->n_iolets;
   double* out = h->d_red + hlb_reduce_partials(h->n) + (K + 1);
-  CUDA_TRY(hlb_launch_reduce(h, h->f[h->cur], h->phase, h->t - 1, h->stepped, monitor, out, h->stream));
+  CUDA_TRY(hlb_launch_reduce(h, h->f[h->cur], h->phase, h->t - 1, h->stepped, totals, monitor, out, h->stream));
   std::vector<double> host((size_t)(1 + 3 * K + 1));  // the monitor's slots without it: left alone
   CUDA_TRY(cudaMemcpyAsync(host.data(), out, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -786,7 +786,7 @@ static int sums_impl(hlb_solver* h, double* mass, double* flux, bool monitor, do
 
 extern "C" int hlb_reduce(hlb_solver* h, double* mass, double* flux) {
   if (!h) return hlb_fail(HLB_ERR_ARG, "null solver");
-  return hlb_no_throw([&] { return sums_impl(h, mass, flux, false, nullptr, nullptr); });
+  return hlb_no_throw([&] { return sums_impl(h, true, mass, flux, false, nullptr, nullptr); });
 }
 
 static int hlb_iolet_monitor_impl(hlb_solver* h, double* flux, double* u_max, double* rho_mean) {
@@ -794,12 +794,9 @@ static int hlb_iolet_monitor_impl(hlb_solver* h, double* flux, double* u_max, do
   if (h->n_iolets == 0 || (!flux && !u_max && !rho_mean)) return HLB_OK;
   const size_t K = (size_t)h->n_iolets;
   std::vector<double> f(K), u(K), r(K);
-  const int rc = sums_impl(h, nullptr, f.data(), true, u.data(), r.data());
-  if (rc == HLB_ERR_DIVERGED && !flux) {
-    // only the flux's caller is told of a run that has blown up
-  } else if (rc) {
-    return rc;
-  }
+  // the flux's caller is told of a run that has blown up; the others need no pass over the whole lattice
+  const int rc = sums_impl(h, flux != nullptr, nullptr, flux ? f.data() : nullptr, true, u.data(), r.data());
+  if (rc) return rc;
   for (size_t k = 0; k < K; ++k) {
     if (flux) flux[k] = f[k];
     if (u_max) u_max[k] = u[k];

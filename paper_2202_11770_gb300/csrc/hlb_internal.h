@@ -215,11 +215,11 @@ cudaError_t hlb_launch_icode(const hlb_solver* h, cudaStream_t s);
 cudaError_t hlb_launch_ctab(const hlb_solver* h, int32_t* misfit, cudaStream_t s);
 // Equilibrium initialisation; u0 [3][n] device or null.
 cudaError_t hlb_launch_init(const hlb_solver* h, void* f, double rho0, const float* u0, cudaStream_t s);
-// Mass (out[0]) and per-iolet flux (out[1..]) in FP64; with `monitor` also
-// after them per iolet max |u| (out[1 + K + k]) and mean rho (out[1 + 2 K + k])
-// over the sites linked to it.
-cudaError_t hlb_launch_reduce(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux, bool monitor,
-                              double* out_dev, cudaStream_t s);
+// With `totals` the mass (out[0]) and per-iolet flux (out[1..]) in FP64, with
+// `monitor` after their places per iolet max |u| (out[1 + K + k]) and mean rho
+// (out[1 + 2 K + k]) over the sites linked to it.
+cudaError_t hlb_launch_reduce(const hlb_solver* h, const void* fin, int mode, int64_t tb, bool have_flux, bool totals,
+                              bool monitor, double* out_dev, cudaStream_t s);
 int64_t hlb_reduce_slots(int64_t n, int32_t n_iolets);
 // Number of per-block mass partials at the start of the reduction scratch.
 int64_t hlb_reduce_partials(int64_t n);
