@@ -551,6 +551,26 @@ __device__ __forceinline__ uint32_t row_offset(int i, uint32_t mask, const uint3
   return ((mask >> (i - 1)) & 1u) ? slot<WIDE>(AAODD ? opp(i) : i, n, s) : slot<WIDE>(AAODD ? i : opp(i), n, pos[CT_GROUPS]);
 }
 
+// Offset-form words of the pair's sites, and the offset that direction i of
+// site x is read from (pull), given the tile's base of the direction.
+__device__ __forceinline__ void load_pair_offsets(const IndexTables& ix, bool wide, uint32_t sn, uint32_t x, uint32_t y,
+                                                  uint32_t* wa, uint32_t* wb) {
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    const uint32_t* row = wide ? ix.ctab + (uint64_t)q * sn : ix.ctab + (uint32_t)q * sn;
+    wa[q] = __ldg(row + x);
+    wb[q] = __ldg(row + y);
+  }
+}
+template <bool WIDE>
+__device__ __forceinline__ uint32_t pair_offset(int i, const uint32_t* w, uint32_t base, uint32_t n, uint32_t x) {
+  const uint32_t o = offset_of(w, i);
+  return o < CT_IOLET ? slot<WIDE>(i, n, base + o) : slot<WIDE>(opp(i), n, x);
+}
+__device__ __forceinline__ bool has_iolet(const IndexTables& ix, uint32_t x) {
+  return (__ldg(ix.imask + (x >> 5)) >> (x & 31)) & 1u;
+}
+
 // Pull A-B step (k_step) with two sites a thread, FP32 or 16-bit storage on the
 // compact table, any number of sites.  Bound by DRAM in FP32 (164 bytes a
 // site with the row-form index) and by instruction issue and latency in 16
@@ -563,8 +583,9 @@ __device__ __forceinline__ uint32_t row_offset(int i, uint32_t mask, const uint3
 // -> 56.4 us, BF16 47.7 -> 38.7 us against one site a thread on it.
 // Prefetch 3 tiles per SM ahead: FP32 495 us with the gathered rows, 500
 // without them, 516 with no prefetch, 537 at 6; 16-bit storage prefetches
-// the index words only.  A tile in offset form takes its sites one by one.
-template <typename S, bool WIDE>
+// the index words only.  A tile in offset form takes its two sites at once as
+// well (TILE_PAIRS; pair_tiles says when), or one after the other.
+template <typename S, bool WIDE, bool TILE_PAIRS>
 __global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_step2(const S* __restrict__ fin, S* __restrict__ fout,
                                                 const IndexTables ix, const LinkRec* __restrict__ links,
                                                 const double* __restrict__ amp, const int32_t* __restrict__ sites,
@@ -607,13 +628,41 @@ __global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_step2(const S* __res
     });
     return;
   }
+  if (TILE_PAIRS) {
+    const uint32_t y1 = y < n ? y : x;
+    uint32_t wa[9], wb[9];
+    bool da = false, db = false;
+    if (x < n) {
+      load_pair_offsets(ix, WIDE, sn, x, y1, wa, wb);
+      da = !has_iolet(ix, x);
+      db = y < n && !has_iolet(ix, y);
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (x >= n) return;
+    const int32_t* tb = ix.tbase + (uint64_t)tile * CT_BASES;
+    float2 h[Q];
+    h[0] = make_float2(ldpop(fin + x), ldpop(fin + y1));
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const uint32_t base = (uint32_t)__ldg(tb + i - 1);
+      h[i] = make_float2(ldpop(at<WIDE>(fin, i, n, pair_offset<WIDE>(i, wa, base, n, x))),
+                         ldpop(at<WIDE>(fin, i, n, pair_offset<WIDE>(i, wb, base, n, y1))));
+    }
+    collide_pair(h, p.omegaf, [&](int i, float2 v) {
+      S* o = i == 0 ? fout + x : at<WIDE>(fout, i, n, slot<WIDE>(i, n, x));
+      if (da) stpop<S>(o, v.x);
+      if (db) stpop<S>(o + 32, v.y);
+    });
+    return;
+  }
   for (uint32_t z = x; z < n && z <= y; z += 32) {
     uint32_t off[Q];
     offset_links<WIDE, LD_NC>(ix, sn, z, tile, [&](int i, bool fluid, uint32_t s) {
       off[i] = fluid ? slot<WIDE>(i, n, s) : slot<WIDE>(opp(i), n, z);
     });
     pdl_wait();
-    if ((__ldg(ix.imask + (z >> 5)) >> (z & 31)) & 1u) continue;
+    if (has_iolet(ix, z)) continue;
     float h[Q];
     h[0] = ldpop(fin + z);
 #pragma unroll
@@ -1232,9 +1281,21 @@ template <typename S>
 uint32_t pair_prefetch(const hlb_solver* h) {
   return sizeof(S) == 4 && h->n < 600000 ? 0u : (uint32_t)h->n_sm * 3u;
 }
-// 16-bit AA odd steps of fewer sites take one site a thread: a wave of the chip
-// holds them all, and the shorter thread is done sooner.
-constexpr int64_t kOddPairSites = 200000;
+// Whether the offset-form tiles of k_step2 (1 to 14 % of a vessel lattice's) take
+// two sites a thread.  us a step, one site after the other / at once: FP32 100k
+// sites 4.28 / 4.97, 150k 5.18 / 5.22, 196k 5.68 / 5.41, 250k 7.08 / 6.52, 600k
+// 16.1 / 14.9; BF16 100k 4.13 / 4.03, 150k 4.74 / 5.29, 196k 5.17 / 5.31, 250k
+// 6.27 / 5.90, 600k 11.0 / 10.5.  Below about a wave of blocks what differs is the
+// trigger: at once, a tile lets the next step's blocks in as soon as it starts,
+// and they settle unevenly on the SMs beside it.
+template <typename S>
+bool pair_tiles(const hlb_solver* h) {
+  return h->n >= (sizeof(S) == 4 ? 175000 : 225000);
+}
+// 16-bit AA odd steps of fewer sites take one site a thread: the shorter thread
+// is done sooner.  BF16, one site / two: 300k sites 9.92 / 10.08 us, 400k 10.95 /
+// 11.01, 600k 13.9 / 13.7.
+constexpr int64_t kOddPairSites = 450000;
 constexpr int64_t kSpreadSites = 4000000;
 inline uint32_t spread_factor(uint32_t iolet, uint32_t blocks) {
   return blocks ? (uint32_t)((((uint64_t)iolet << 32) + blocks - 1) / blocks) : 0u;
@@ -1282,7 +1343,9 @@ cudaError_t launch_gather(const hlb_solver* h, const void* fin, void* fout, cons
       const unsigned grid = whole ? spread_iolets(h, CT_TILE, PAIR, &spread)
                                   : spread_evenly(ntiles, iolets ? iolet_blocks(h, PAIR) : 0u, &spread);
       if (grid == 0) return cudaSuccess;
-      return launch_pdl(h->off32 ? k_step2<S, false> : k_step2<S, true>, grid, PAIR, s, (const S*)fin, (S*)fout, h->index(),
+      auto kernel = pair_tiles<S>(h) ? (h->off32 ? k_step2<S, false, true> : k_step2<S, true, true>)
+                                     : (h->off32 ? k_step2<S, false, false> : k_step2<S, true, false>);
+      return launch_pdl(kernel, grid, PAIR, s, (const S*)fin, (S*)fout, h->index(),
                         h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, spread, pair_prefetch<S>(h), tile0, p);
     }
   }
