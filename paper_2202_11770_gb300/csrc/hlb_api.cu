@@ -246,7 +246,7 @@ Layout layout(const hlb_lattice* L, const hlb_options* o, const std::vector<int6
   y.tbase = off; off += align_up(sizeof(int32_t) * hlb::CT_BASES * (size_t)((n + hlb::CT_TILE - 1) / hlb::CT_TILE));
   y.rtab = off; off += align_up(sizeof(uint32_t) * hlb::CT_ROW_WORDS * (size_t)row_stride(n));
   y.rbase = off; off += align_up(sizeof(int32_t) * hlb::CT_GROUPS * (size_t)((n + hlb::CT_TILE - 1) / hlb::CT_TILE));
-  y.ctflag = off; off += align_up(sizeof(int32_t));
+  y.ctflag = off; off += align_up(2 * sizeof(int32_t));
   y.links = off; off += align_up(sizeof(LinkRec) * (size_t)std::max<int64_t>(y.n_links, 1));
   y.amp = off; off += align_up(sizeof(double) * (size_t)std::max(y.n_groups, 1));
   y.ampf = off; off += align_up(sizeof(float) * (size_t)std::max(y.n_groups, 1));
@@ -505,10 +505,10 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   if (e == cudaSuccess && y.n_links > 0) e = hlb_launch_recode(h, st);
   // compact index table from the re-coded one; the fit flag comes back with
   // the final synchronisation
-  int32_t misfit = 1;
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_misfit, 0, sizeof(int32_t), st);
+  int32_t misfit[2] = {1, 0};  // a span that does not fit, tiles in offset form
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_misfit, 0, sizeof misfit, st);
   if (e == cudaSuccess) e = hlb_launch_ctab(h, d_misfit, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&misfit, d_misfit, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(misfit, d_misfit, sizeof misfit, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_amp, ampf.data(), sizeof(double) * ampf.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_ampf, 0, sizeof(float) * ampf.size(), st);
   if (e == cudaSuccess && h->d_normal)
@@ -554,7 +554,8 @@ static int create_impl(const hlb_lattice* L, const hlb_options* o, void* ws, siz
   if (e == cudaSuccess) e = cudaMemsetAsync(h->f[0], 0, h->state_bytes(), st);  // rest: h = f - w = 0
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return hlb_cuda_fail(e, "hlb_create upload");  // the owner frees h
-  h->compact = !o->full_index && misfit == 0;
+  h->compact = !o->full_index && misfit[0] == 0;
+  h->offset_major = misfit[1] > (n + CT_TILE - 1) / CT_TILE / 2;
   h->cur = 0;
   h->phase = 0;
   h->t = 0;

@@ -64,9 +64,11 @@ __device__ __forceinline__ void l2_prefetch(const void* q, uint32_t bytes) {
 // 9-26: for direction i = lane - 8, the population row its gathers read
 // (ROWOPP: row opp(i), as the AA odd step reads; else row i) from the
 // tile's smallest source for i, 320 sites wide (the sources of a tile span
-// about 255 sites on vessel lattices).  A tile in offset form is left to its
-// own loads.  Every range is clamped to its array: rtab holds CT_ROW_WORDS
-// rows of sn words, A 19 rows of n populations.
+// about 255 sites on vessel lattices).  A tile in the form that is rare in its
+// lattice is left to its own loads: where most tiles have the offset form, the
+// index words are its nine rows (lanes 0-8) and the bases its own.  Every range
+// is clamped to its array: rtab holds CT_ROW_WORDS rows of sn words, ctab nine,
+// A 19 rows of n populations.
 template <typename S, bool POPS, bool ROWOPP>
 __device__ __forceinline__ void prefetch_tile(const S* A, const IndexTables& ix, uint32_t n, uint32_t sn,
                                               uint32_t tile) {
@@ -74,16 +76,17 @@ __device__ __forceinline__ void prefetch_tile(const S* A, const IndexTables& ix,
   const int l = threadIdx.x & 31;
   if (tile >= ntiles) return;
   const uint64_t x0 = (uint64_t)tile * BLOCK;
-  if (l < CT_ROW_WORDS) {
+  if (l < (ix.offset_major ? (Q - 1) / 2 : CT_ROW_WORDS)) {
     const uint64_t e = x0 + BLOCK < (uint64_t)sn ? x0 + BLOCK : (uint64_t)sn;  // sn: a multiple of 4
-    l2_prefetch(ix.rtab + (uint64_t)l * sn + x0, (uint32_t)((e - x0) * 4));
+    l2_prefetch((ix.offset_major ? ix.ctab : ix.rtab) + (uint64_t)l * sn + x0, (uint32_t)((e - x0) * 4));
   } else if (POPS && l >= 9 && l < 9 + Q - 1) {
     const int i = l - 8, y = k_cy[i], z = k_cz[i];
     const int32_t* rb = ix.rbase + (uint64_t)tile * CT_GROUPS;
-    if (__ldg(rb) == CT_NO_ROWS) return;
+    if ((__ldg(rb) == CT_NO_ROWS) != (ix.offset_major != 0)) return;
     // row_group(i) of a run-time direction
     const int g = z == 0 ? (y > 0 ? 0 : 1) : (y == 0 ? (z > 0 ? 2 : 3) : (z > 0 ? (y > 0 ? 4 : 7) : (y > 0 ? 6 : 5)));
-    const int64_t first = (int64_t)x0 - k_cx[i] + ((y | z) ? __ldg(rb + g) : 0);
+    const int64_t first = ix.offset_major ? __ldg(ix.tbase + (uint64_t)tile * CT_BASES + (i - 1))
+                                          : (int64_t)x0 - k_cx[i] + ((y | z) ? __ldg(rb + g) : 0);
     const uint64_t b = first > 0 ? (uint64_t)first : 0;
     const uint64_t r = ROWOPP ? (uint64_t)lane_opp(i) : (uint64_t)i;
     const uint64_t e = b + 320 < (uint64_t)n ? b + 320 : (uint64_t)n;
@@ -777,8 +780,11 @@ __global__ void __launch_bounds__(256, 8) k_aa_fix(S* A, const int32_t* __restri
 // post-collision population into the slot it came from, where the site
 // downstream (or, across a wall or iolet, the site itself) reads it in the
 // next (even) step.  Sites with iolet links: aa_iolet_site or k_aa_fix.
-// This one-site form serves FP64 storage and the int32 table; k_aa_odd2 the
-// rest.  The 18 slot offsets (32-bit) are computed once and held in registers
+// This one-site form serves FP64 storage, the int32 table, small 16-bit
+// lattices (kOddPairSites) and, in 16 bits or from kOffsetPairSites on, those
+// whose tiles mostly have the offset form (2.0M sites in (x, y, z) order, BF16:
+// 41 us; k_aa_odd2 44, and 47 with both sites at once, which spills); k_aa_odd2
+// the rest.  The 18 slot offsets (32-bit) are computed once and held in registers
 // for the stores, so the index row is read once.  WIDE: offsets within
 // direction pairs (lattices above ~226M sites), four blocks per SM instead
 // of five.  CT: codes from the compact index table, and the first warp
@@ -986,6 +992,7 @@ __global__ void __launch_bounds__(CT_TILE, 3) k_ctab_build(const int32_t* __rest
     if (threadIdx.x == 0) {
       tbase[(int64_t)blockIdx.x * CT_BASES + (i - 1)] = (int32_t)b;
       if (any && hi - lo > CT_MAX_SPAN) atomicOr(misfit, 1);
+      if (i == 1) atomicAdd(misfit + 1, 1);
     }
     const uint32_t o = s[i] >= 0 ? ((uint32_t)s[i] - b) & 0xffffu : (s[i] == -1 ? CT_WALL : CT_IOLET);
     if (i & 1) {
@@ -1290,12 +1297,16 @@ uint32_t pair_prefetch(const hlb_solver* h) {
 // and they settle unevenly on the SMs beside it.
 template <typename S>
 bool pair_tiles(const hlb_solver* h) {
-  return h->n >= (sizeof(S) == 4 ? 175000 : 225000);
+  return h->offset_major || h->n >= (sizeof(S) == 4 ? 175000 : 225000);
 }
 // 16-bit AA odd steps of fewer sites take one site a thread: the shorter thread
 // is done sooner.  BF16, one site / two: 300k sites 9.92 / 10.08 us, 400k 10.95 /
 // 11.01, 600k 13.9 / 13.7.
 constexpr int64_t kOddPairSites = 450000;
+// FP32 AA steps of fewer sites take two sites a thread in offset form too, their
+// iolet sites in the grid: (x, y, z) order 50k sites 4.1 us against 5.5 (one site
+// a thread and the pass), 500k 13.5 / 15.3, 2.0M 62.5 / 59.8, 8.0M 245 / 224.
+constexpr int64_t kOffsetPairSites = 1000000;
 constexpr int64_t kSpreadSites = 4000000;
 inline uint32_t spread_factor(uint32_t iolet, uint32_t blocks) {
   return blocks ? (uint32_t)((((uint64_t)iolet << 32) + blocks - 1) / blocks) : 0u;
@@ -1386,7 +1397,7 @@ struct StepRangeOp {
 // 38.6 / 38.2, 20M 345 / 312) and keeps the pass, as FP64 and the int32 table do.
 template <typename S>
 bool aa_in_grid(const hlb_solver* h) {
-  return sizeof(S) == 4 && h->compact && h->n < 4000000;
+  return sizeof(S) == 4 && h->compact && h->n < (h->offset_major ? kOffsetPairSites : 4000000);
 }
 
 // The iolet blocks of a grid with `bulk` bulk blocks of `threads` threads.
@@ -1402,15 +1413,15 @@ cudaError_t launch_aa(const hlb_solver* h, S* A, bool odd, const StepParams& p, 
   const unsigned g = grid_for(h->n);
   if (odd) {
     if constexpr (sizeof(S) <= 4) {
-      if (h->compact && (sizeof(S) == 4 || h->n >= kOddPairSites)) {
+      if (h->compact && (sizeof(S) == 4 ? !h->offset_major || h->n < kOffsetPairSites
+                                        : !h->offset_major && h->n >= kOddPairSites)) {
         const AAIolets io = aa_iolets<GRID>(h, g, PAIR);
         return launch_pdl(h->off32 ? k_aa_odd2<S, false, GRID> : k_aa_odd2<S, true, GRID>, g + io.blocks, PAIR, s, A,
                           h->index(), io, pair_prefetch<S>(h), p);
       }
     }
     if constexpr (!GRID) {
-      constexpr bool CT = sizeof(S) != 4;  // FP32 takes two sites a thread
-      return launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, CT> : k_aa_odd<S, true, CT>)
+      return launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, true> : k_aa_odd<S, true, true>)
                                    : (h->off32 ? k_aa_odd<S, false, false> : k_aa_odd<S, true, false>),
                         g, BLOCK, s, A, h->index(), (uint32_t)h->n_sm * (h->off32 ? 3u : 4u), p);
     }

@@ -74,6 +74,7 @@ struct hlb_solver {
   uint32_t* d_rtab = nullptr;
   int32_t* d_rbase = nullptr;
   bool compact = false;               // bulk step and adjoint codes from the compact table
+  bool offset_major = false;          // more than half of its tiles have the offset form (sites not in (z, y, x) order)
   hlb::LinkRec* d_links = nullptr;
   double* d_amp = nullptr;            // [n_groups_total]
   float* d_ampf = nullptr;            // [n_groups_total] the same rounded to float (FP32 kernels)
@@ -112,7 +113,7 @@ struct hlb_solver {
   int64_t n_ilist = 0;                // entries of d_ilist
   int64_t red_slots = 0;
 
-  hlb::IndexTables index() const { return {d_src, d_ctab, d_tbase, d_rtab, d_rbase, d_imask}; }
+  hlb::IndexTables index() const { return {d_src, d_ctab, d_tbase, d_rtab, d_rbase, d_imask, offset_major ? 1 : 0}; }
   size_t elem_bytes() const;
   size_t state_bytes() const { return elem_bytes() * 19 * (size_t)n; }
   // kernel parameters for a launch that gathers with boundary data at time tb

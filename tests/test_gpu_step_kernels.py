@@ -94,3 +94,22 @@ def test_trees(prec, scheme, sites):
     assert lat.n % 256
     for wide in (False, True) if sites < 1_000_000 else (False,):
         _same(lat, prec, scheme, sites, wide)
+
+
+@pytest.mark.parametrize("order", ["x, y, z", "backwards"])
+@pytest.mark.parametrize("sites", [3_000, 49_000, 470_000])
+def test_sites_in_another_order(sites, order):
+    """Lattices whose tiles have the offset form throughout: their own kernels'
+    choice and prefetch, in both schemes and every storage."""
+    base = geo.tree(2, 2202, target_sites=sites, length_ratio=5.0)
+    x, y, z = base.xyz.T
+    perm = np.lexsort((z, y, x)) if order == "x, y, z" else np.arange(base.n)[::-1]
+    inv = np.empty(base.n, np.int64)
+    inv[perm] = np.arange(base.n)
+    src = base.src[:, perm]
+    lat = geo.from_arrays(base.xyz[perm], np.where(src >= 0, inv[np.maximum(src, 0)], src), iolets=base.iolets,
+                          wall_normal=base.wall_normal[:, perm], amp_group=base.amp_group[perm])
+    for prec in ("fp32", "bf16", "fp16", "fp64"):
+        for scheme in ("ab", "aa"):
+            for wide in (False, True):
+                _same(lat, prec, scheme, sites, wide)
