@@ -1489,7 +1489,11 @@ __global__ void __launch_bounds__(BLOCK) k_wk_update(const S* __restrict__ fin, 
                                                      const double* __restrict__ par, double* __restrict__ state,
                                                      double* ioval, double* __restrict__ iovnext, int shift) {
   using R = typename Real<S>::type;
-  __shared__ double sh[BLOCK / 32], mass[BLOCK];
+  // Links between two block barriers.  FP32 AA steps of 50k sites with outlets 7.9
+  // us at two a thread, 8.3 at one; at four (8 KB) the FP64 pull step, which lasts
+  // as long as the SM that gets most blocks, took 50 to 70 us instead of 42.
+  constexpr int CHUNK = 2 * BLOCK;
+  __shared__ double sh[BLOCK / 32], mass[CHUNK];
   const int k = blockIdx.x;
   pdl_wait();
   pdl_trigger();
@@ -1500,36 +1504,30 @@ __global__ void __launch_bounds__(BLOCK) k_wk_update(const S* __restrict__ fin, 
   }
   const int64_t n = p.n;
   double acc = 0;
-  for (int64_t r0 = begin[k], end = begin[k + 1]; r0 < end; r0 += BLOCK) {
-    const int64_t r = r0 + threadIdx.x;
-    if (r >= end) {
-      mass[threadIdx.x] = 0;
-    } else if (AA) {
-      mass[threadIdx.x] = lflux[r];
-    } else {
+  for (int64_t r0 = begin[k], end = begin[k + 1]; r0 < end; r0 += CHUNK) {
+    const int count = (int)min((int64_t)CHUNK, end - r0);
+    for (int m = threadIdx.x; m < count; m += BLOCK) {
+      const int64_t r = r0 + m;
+      if (AA) {
+        mass[m] = lflux[r];
+        continue;
+      }
       const LinkRec L = links[r];
       const int64_t x = L.site;
       R own[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) own[i] = ldpop(fin + (int64_t)i * n + x);
       const Macro<R> ms = moments<R>(own);
-      const int j = L.dir;
-      R out = R(0), val = R(0);
-#pragma unroll
-      for (int i = 1; i < Q; ++i)
-        if (i == opp(j)) out = own[i];
-#pragma unroll
-      for (int i = 1; i < Q; ++i)
-        if (i == j) val = iolet_value<R>(i, L, out, ms.rho, ms.ux, ms.uy, ms.uz, amp, p);
-      mass[threadIdx.x] = (double)val - (double)out;
+      const R out = ldpop(fin + (int64_t)lane_opp(L.dir) * n + x);
+      const R a = BC<R>::amp(p, amp, L.kind == 0 && L.group >= 0 ? L.group : 0);
+      const R val = lane_iolet_value<R>(L.dir, L, out, ms.rho, ms.ux, ms.uy, ms.uz, a, BC<R>::val(p, L.iolet), p);
+      mass[m] = (double)val - (double)out;
     }
-    // in the order of a multi-step launch's outlet blocks (hlb_multi.cu); the zeros past the end add nothing
+    // in the order of a multi-step launch's outlet blocks (hlb_multi.cu)
     __syncthreads();
-    if (threadIdx.x < kWkLanes) {
-#pragma unroll
-      for (int u = 0; u < BLOCK / kWkLanes; ++u) acc += mass[threadIdx.x + u * kWkLanes];
-    }
-    __syncthreads();
+    if (threadIdx.x < kWkLanes)
+      for (int m = threadIdx.x; m < count; m += kWkLanes) acc += mass[m];
+    if (r0 + CHUNK < end) __syncthreads();
   }
   const double flux = block_sum(acc, sh);
   if (threadIdx.x == 0) {
