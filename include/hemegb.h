@@ -108,10 +108,10 @@ typedef struct {
 
 /* precision: HLB_FP32 / HLB_BF16 / HLB_FP16 / HLB_FP64 storage.
  * scheme: HLB_PULL_AB (two population buffers, pull gather) or HLB_AA
- *   (one buffer, alternating in-place even/odd steps); AUTO picks the
- *   scheme measured faster for the lattice size: pull A-B below 750k sites
- *   (one launch per step; such states fit in the GPU's L2 cache), AA from
- *   750k sites on (fewer bytes per site).
+ *   (one buffer, alternating in-place even/odd steps); AUTO picks by the
+ *   lattice size: pull A-B below 750k sites (one launch per step; such states
+ *   fit in the GPU's L2 cache), AA from 750k sites on (half of the population
+ *   memory, fewer bytes per site).
  * ladd_rho_one: 1 = use rho = 1 in the Ladd correction instead of the
  *   site's density (the paper does not say which density).
  * ghost_full_u: 1 = pressure-iolet ghost velocity u instead of (u.n) n.
@@ -209,7 +209,8 @@ int hlb_set_pressure(hlb_solver* h, int32_t k, const hlb_waveform* w);
  * q being the outflow (minus the mass flux of hlb_reduce) of the step that
  * produced the current state; C = 0 is a pure resistance, ghost density
  * rho_d + (Rp + Rd) q.  The coupling is explicit (one step of lag) and runs
- * one extra small kernel per step.  rho_c starts at rho_c0 (C > 0) and the
+ * one extra small kernel per step, or inside a multi-step launch (hlb_step)
+ * with the same results.  rho_c starts at rho_c0 (C > 0) and the
  * outflow history at 0; hlb_init_equilibrium clears the history again.
  * Densities are lattice densities (pressure = rho / 3).  HLB_ERR_ARG if k
  * is not a pressure iolet, a parameter is negative, rho_d or rho_c0 is not
@@ -233,7 +234,8 @@ int hlb_init_equilibrium(hlb_solver* h, double rho0, const float* u0, int32_t wh
  * stream capture.  Its blocks pass populations to one another with waits that
  * are bounded: should one run out, the state is no longer valid, and every
  * synchronising call returns HLB_ERR_WAIT until hlb_init_equilibrium or
- * hlb_set_state sets a new one (device outputs hold NaN). */
+ * hlb_set_state sets a new one (device outputs hold NaN, and so may the models
+ * of Windkessel outlets: hlb_set_windkessel sets them anew). */
 int hlb_step(hlb_solver* h, int64_t n);
 int hlb_time(const hlb_solver* h, int64_t* t);
 

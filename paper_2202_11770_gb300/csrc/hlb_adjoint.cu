@@ -421,8 +421,8 @@ __device__ __forceinline__ typename Real<S>::type adjoint_iolet_site(const S* __
 }
 
 // One reverse step in one launch.  Every stride-th block (the first
-// n_iolet_blocks of them) takes eight iolet sites, a warp each; the others
-// take 256 bulk sites, a thread each.  Spreading the short, latency-bound
+// n_iolet_blocks of them) takes four iolet sites, a warp each; the others
+// take 128 bulk sites, a thread each.  Spreading the short, latency-bound
 // iolet blocks through the grid lets them run beside the bulk blocks instead
 // of ahead of them.  Block b's dJ/dtau partial goes to part[b] (fixed order).
 // WIDE: offsets within direction pairs (lattices above ~226M sites); the

@@ -216,13 +216,15 @@ int validate(const hlb_lattice* L, const hlb_options* o, std::vector<int64_t>* p
   return HLB_OK;
 }
 
-// AUTO resolves by lattice size.  The AA pattern moves 158 B per FP32 site
-// update against 164 B for pull A-B (row-form index) and needs one buffer
-// instead of two.  Measured per step (seeded vessel trees), pull A-B / AA: FP32
-// 0.5M sites 12.7 / 13.0 us (the state fits in L2), 1.0M 29.7 / 23.6, 2.0M 56.1
-// / 54.9, 8.0M 204 / 210, 20M 484 / 492; BF16 0.5M 9.7 / 13.0, 1.0M 18.7 / 20.3,
-// 2.0M 38.7 / 38.2, 20M 343 / 311.  AA from 750k sites: at large FP32 lattices it
-// gives up 2-3 % for half of the population memory.
+// AUTO resolves by lattice size alone, so that a lattice's scheme (and memory) is
+// the same in every precision.  The AA pattern moves 158 B per FP32 site update
+// against 164 B for pull A-B (row-form index) and needs one buffer instead of
+// two.  Measured per step (seeded vessel trees), pull A-B / AA: FP32 0.4M sites
+// 8.6 / 10.4 us and 0.6M 14.9 / 14.6 (the state fits in L2), 1.0M 27.7 / 23.7, 1.5M
+// 40.5 / 40.3, 2.0M 55.2 / 54.5, 8.0M 204 / 210, 20M 484 / 492; BF16 0.6M 10.5 /
+// 13.9, 1.0M 17.3 / 20.1, 1.5M 29.5 / 26.2, 2.0M 38.9 / 38.4, 20M 343 / 311.  AA from
+// 750k sites: that is where FP32 gains; 16-bit storage gives up 16 % up to about
+// 1.2M sites, large FP32 lattices 2-3 %, for half of the population memory.
 constexpr int64_t AA_MIN_SITES = 750000;
 int32_t resolve_scheme(int32_t scheme, int64_t n) {
   if (scheme != HLB_SCHEME_AUTO) return scheme;

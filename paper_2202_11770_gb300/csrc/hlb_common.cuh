@@ -76,8 +76,6 @@ template <typename S>
 __device__ __forceinline__ typename Real<S>::type ldpop(const S* p) {
   return to_real(__ldg(p));
 }
-// Streaming load of the index table (read once per step, evict first).
-__device__ __forceinline__ int32_t ldidx(const int32_t* p) { return __ldcs(p); }
 // Streaming store of a population (next read is a full sweep later).
 template <typename S>
 __device__ __forceinline__ void stpop(S* p, typename Real<S>::type v) {
@@ -616,12 +614,12 @@ struct IndexTables {
   int32_t offset_major;   // more than half of the tiles have the offset form: what a prefetch goes by
 };
 
-// How a kernel loads its index entries: read-only cached, streaming (read
-// once, evict first), or cached in L1 for a re-read by the same thread.
-enum { LD_NC = 0, LD_STREAM = 1, LD_L1 = 2 };
+// How a kernel loads its index entries: read-only cached, or streaming (read
+// once, evict first).
+enum { LD_NC = 0, LD_STREAM = 1 };
 template <int LD, typename T>
 __device__ __forceinline__ T ld_index(const T* p) {
-  return LD == LD_STREAM ? __ldcs(p) : (LD == LD_L1 ? __ldca(p) : __ldg(p));
+  return LD == LD_STREAM ? __ldcs(p) : __ldg(p);
 }
 
 // The offset-form entries of site x: w[9] from ctab, b[i - 1] the tile's bases.

@@ -16,9 +16,9 @@
 //    write the results to the very same 19 slots.  152 B (even) + 164 B
 //    (odd; 224 B with the int32 table) per FP32 update.
 //
-// The bulk kernels take the index from its compact form (hlb_common.cuh,
-// built by k_ctab_build) unless the lattice does not fit it; iolet-site
-// paths and read-back kernels use the int32 table.
+// The bulk and read-back kernels take the index from its compact form
+// (hlb_common.cuh, built by k_ctab_build) unless the lattice does not fit it;
+// iolet-site paths, and what reads single sites, use the int32 table.
 //
 // Read modes of the readback kernels: LOCAL (the buffer holds f(t) in place),
 // GATHER_AB (the buffer holds s'(t-1); boundaries applied while gathering),

@@ -159,7 +159,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
 // ---- many steps a launch (hlb_multi.cu) ----
 constexpr int kMultiVals = 2048;           // boundary values [step][iolet] of a launch
 constexpr int kMultiMin = 4;               // fewer steps are launched one by one
-constexpr int64_t kMultiSites = 24000;     // sites up to which it is the faster form (hlb_multi_steps)
+constexpr int64_t kMultiSites = 24000;     // sites up to which FP32 and 16-bit steps use it (hlb_multi_steps)
 constexpr int64_t kMultiMaxSites = 100000; // sites of a lattice that may fit on the device at once
 // 64-bit words of device scratch.
 size_t hlb_multi_words(int64_t n, int64_t n_links, int32_t n_iolets, int32_t precision);

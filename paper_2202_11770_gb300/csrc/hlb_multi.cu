@@ -9,7 +9,7 @@
 // produced it (FP64: two words, half a value each).  A reader polls the word
 // itself, so a step costs one trip to L2 and back: no barrier, no fence, no
 // flag.  A grid of flags with a release and an acquire a step measured 3.8 us
-// a step at 12k sites, slower than the launches.
+// a step at 12k sites, slower than the launches (this form: 2.4).
 //
 // Two word buffers, by step parity.  A site overwrites the words of step k - 1
 // at step k + 1, after it has read step k of every site it pulls from; those
@@ -482,13 +482,14 @@ int hlb_multi_blocks(const hlb_solver* h) {
 
 // The pull scheme on the compact table with mutual links, all blocks resident,
 // enough steps, and outside a stream capture (where the step-by-step launches
-// were and stay what is captured).  Up to kMultiSites sites, measured per step
-// against a launch: 2.6 against 3.4 us at 12k sites, 3.4 against 3.5 at 30k,
-// 3.8 against 3.6 at 50k (18 words of 8 bytes a site through L2).  FP64 runs
-// at the rate of its arithmetic, spread over more SMs by the smaller blocks:
-// 11.6 against 20 us at 12k, 27 against 29 at 50k, so whatever fits.  With
-// Windkessel outlets a step is two launches, the second a chain of loads:
-// 6.5 against 12.3 us at 50k, so whatever fits as well.
+// were and stay what is captured).  FP32 and 16 bits up to kMultiSites, where the
+// two forms are about to cross: 2.4 us a step against 3.2-3.4 at 12k sites, 2.7 /
+// 3.3 at 18k, 3.1 / 3.35 at 24k; at 50k 3.8 / 3.6 (18 words of 8 bytes a site go
+// through L2).  FP64 runs at the rate of its arithmetic, spread over more SMs by
+// the smaller blocks, 10.2 against 19.8 us at 12k and 14.1 / 19.3 at 24k, so
+// whatever fits (about 36k sites).  With Windkessel outlets a step is two
+// launches, the second a chain of loads, 7.8 against 10.6 us at 50k, so whatever
+// fits as well.
 int hlb_multi_steps(const hlb_solver* h, int64_t left) {
   if (h->multi_blocks == 0 || !h->compact || !h->off32 || left < kMultiMin) return 0;
   if (h->n > kMultiSites && h->precision != HLB_FP64 && !h->any_wk()) return 0;
