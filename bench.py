@@ -226,10 +226,25 @@ def time_form(lat, precision, scheme, steps, warmup, torch, dist=None, tau=0.55,
     return total, durs, t_first, compact
 
 
-def kernel_names(n, compact=True, wide=False):
-    """Names of the step kernels the library launches (pull A-B, AA odd step):
-    the pull step takes two sites a thread (k_step2) on the compact table
-    with 32-bit offsets when the site count is even."""
+# Site counts of the library's launch rules (csrc/hlb_forward.cu): FP32 AA steps
+# of fewer sites step their iolet sites in the grid, 16-bit AA odd steps of fewer
+# take one site a thread.
+AA_IN_GRID_SITES = 4_000_000
+ODD_PAIR_SITES = 450_000
+
+
+def kernel_names(n, compact=True, wide=False, precision="fp32"):
+    """Names of the step kernels (pull A-B, AA odd step) that the library
+    launches on a lattice in (z, y, x) order.  On the compact table with its
+    row form (compact = "rows"): two sites a thread in FP32 and 16 bits, any
+    site count and offset width, but one in the AA odd step of small 16-bit
+    lattices and in FP64.  For a table of 16-bit offsets alone (True) or the
+    int32 table (False): two in the pull step of even site counts with 32-bit
+    offsets."""
+    if compact == "rows":
+        pair = precision != "fp64"
+        return ("k_step2" if pair else "k_step",
+                "k_aa_odd2" if pair and (precision == "fp32" or n >= ODD_PAIR_SITES) else "k_aa_odd")
     return ("k_step2" if compact and not wide and n % 2 == 0 else "k_step", "k_aa_odd")
 
 
@@ -238,7 +253,7 @@ def form_stats(lat, precision, scheme, total, durs, t_first, steps, peak, compac
     (CUDA events around every step: each step is one kernel launch).
     compact: False, True (offset form) or "rows" (row form of the table)."""
     n = lat.n
-    k_ab, k_odd = kernel_names(n, compact)
+    k_ab, k_odd = kernel_names(n, compact, precision=precision)
     e = ELEM[precision]
     out = {"scheme": scheme, "mlups": n * steps / (total * 1e-3) / 1e6, "ms_per_step": total / steps,
            "index": "compact" if compact else "int32"}
@@ -625,14 +640,14 @@ def run_ours(args):
     ms, total_updates = aggregate_ranks(ms, n * args.steps, dist, "cuda")
     value = total_updates / (ms * 1e-3) / 1e6
     head = form_stats(lat, prec0, scheme, ms, durs, t_first, args.steps, peak, "rows" if compact else False)
-    kname = kernel_names(n, compact, args.wide_offsets)[0 if scheme == "ab" else 1]
+    kname = kernel_names(n, "rows" if compact else False, precision=prec0)[0 if scheme == "ab" else 1]
     kst = head["kernels"][kname]
     traffic = None
     # the recorded bytes belong to the 32-bit-offset kernels (lattices below
     # ~226M sites without --wide-offsets); larger lattices run the wide form
     off32 = not args.wide_offsets and 19 * ((n + 3) // 4 * 4) <= 0xFFFFFFFF
     if (TRAFFIC["sha"] == kernel_sha() and TRAFFIC["index"] == ("compact" if compact else "int32") and off32
-            and kname in TRAFFIC["bytes_per_site"]):
+            and prec0 == "fp32" and kname in TRAFFIC["bytes_per_site"]):
         traffic = TRAFFIC["bytes_per_site"][kname] * n
 
     forms = {f"{prec0}_{scheme}": head}
@@ -680,9 +695,7 @@ def run_ours(args):
                        "fill": round(lat.info["fill"], 4)},
             "roofline": {"bound": "hbm", "achieved": kst["gbs"], "peak": peak, "unit": "GB/s",
                          "frac": kst["gbs"] / peak, "traffic": traffic, "peak_kind": peak_kind,
-                         # FP32 and 16-bit storage on the compact table: the two-site kernels
-                         "kernel": (f"{kname.rstrip('2')}{'2' if compact and ELEM[prec0] <= 4 else ''}"
-                                    f"<{CTYPE[prec0]}>"), "launches": kst["launches"], "mean_us": kst["mean_us"],
+                         "kernel": f"{kname}<{CTYPE[prec0]}>", "launches": kst["launches"], "mean_us": kst["mean_us"],
                          "timed": "CUDA events around each step" + (
                              " (odd step = the kernel + the k_aa_fix pass)" if scheme == "aa" else ""),
                          "algorithmic_bytes_per_site": kst["bytes_per_site"],
@@ -692,7 +705,7 @@ def run_ours(args):
             "clocks": clk,
             # per step: the fused kernel, plus the iolet pass of an AA step on a large lattice
             "gpu_launches": args.steps * (2 if scheme == "aa" and bool((lat.src <= -2).any()) and not (
-                compact and prec0 == "fp32" and n < 4_000_000) else 1),
+                compact and prec0 == "fp32" and n < AA_IN_GRID_SITES) else 1),
             "forms": forms,
             "precision_vs_oracle": precision,
             "adjoint": adjoint,
