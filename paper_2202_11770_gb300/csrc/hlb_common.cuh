@@ -611,7 +611,6 @@ struct IndexTables {
   const uint32_t* rtab;   // [CT_ROW_WORDS][sn] row form
   const int32_t* rbase;   // [tiles][CT_GROUPS]
   const uint32_t* imask;  // [(n + 31) / 32] bit x % 32 of word x / 32: site x has an iolet link
-  int32_t offset_major;   // more than half of the tiles have the offset form: what a prefetch goes by
 };
 
 // How a kernel loads its index entries: read-only cached, or streaming (read

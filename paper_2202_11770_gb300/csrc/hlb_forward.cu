@@ -66,26 +66,30 @@ __device__ __forceinline__ void l2_prefetch(const void* q, uint32_t bytes) {
 // tile's smallest source for i, 320 sites wide (the sources of a tile span
 // about 255 sites on vessel lattices).  A tile in the form that is rare in its
 // lattice is left to its own loads: where most tiles have the offset form, the
-// index words are its nine rows (lanes 0-8) and the bases its own.  Every range
-// is clamped to its array: rtab holds CT_ROW_WORDS rows of sn words, ctab nine,
+// index words are its nine rows (lanes 0-8) and the bases its own (kPrefetchOffsets
+// in `pf`; OFFSETS: asked at all, which the small-lattice form of k_step2 is not:
+// the longer code made some of its steps 3 to 10 % slower).  Every range is clamped to its array: rtab holds CT_ROW_WORDS rows of sn words, ctab nine,
 // A 19 rows of n populations.
-template <typename S, bool POPS, bool ROWOPP>
+constexpr uint32_t kPrefetchOffsets = 0x80000000u;
+template <typename S, bool POPS, bool ROWOPP, bool OFFSETS>
 __device__ __forceinline__ void prefetch_tile(const S* A, const IndexTables& ix, uint32_t n, uint32_t sn,
-                                              uint32_t tile) {
+                                              uint32_t tile, uint32_t pf) {
+  const bool offsets = OFFSETS && (pf & kPrefetchOffsets);
+  tile += pf & ~kPrefetchOffsets;
   const uint32_t ntiles = (n + BLOCK - 1) / BLOCK;
   const int l = threadIdx.x & 31;
   if (tile >= ntiles) return;
   const uint64_t x0 = (uint64_t)tile * BLOCK;
-  if (l < (ix.offset_major ? (Q - 1) / 2 : CT_ROW_WORDS)) {
+  if (l < (offsets ? (Q - 1) / 2 : CT_ROW_WORDS)) {
     const uint64_t e = x0 + BLOCK < (uint64_t)sn ? x0 + BLOCK : (uint64_t)sn;  // sn: a multiple of 4
-    l2_prefetch((ix.offset_major ? ix.ctab : ix.rtab) + (uint64_t)l * sn + x0, (uint32_t)((e - x0) * 4));
+    l2_prefetch((offsets ? ix.ctab : ix.rtab) + (uint64_t)l * sn + x0, (uint32_t)((e - x0) * 4));
   } else if (POPS && l >= 9 && l < 9 + Q - 1) {
     const int i = l - 8, y = k_cy[i], z = k_cz[i];
     const int32_t* rb = ix.rbase + (uint64_t)tile * CT_GROUPS;
-    if ((__ldg(rb) == CT_NO_ROWS) != (ix.offset_major != 0)) return;
+    if ((__ldg(rb) == CT_NO_ROWS) != offsets) return;
     // row_group(i) of a run-time direction
     const int g = z == 0 ? (y > 0 ? 0 : 1) : (y == 0 ? (z > 0 ? 2 : 3) : (z > 0 ? (y > 0 ? 4 : 7) : (y > 0 ? 6 : 5)));
-    const int64_t first = ix.offset_major ? __ldg(ix.tbase + (uint64_t)tile * CT_BASES + (i - 1))
+    const int64_t first = offsets ? __ldg(ix.tbase + (uint64_t)tile * CT_BASES + (i - 1))
                                           : (int64_t)x0 - k_cx[i] + ((y | z) ? __ldg(rb + g) : 0);
     const uint64_t b = first > 0 ? (uint64_t)first : 0;
     const uint64_t r = ROWOPP ? (uint64_t)lane_opp(i) : (uint64_t)i;
@@ -216,7 +220,7 @@ __global__ void __launch_bounds__(BLOCK, 5) k_step(const S* __restrict__ fin, S*
   if (tile0 == kNoTile) return;
   const uint32_t tile = tile0 + j;
   const uint32_t x = tile * BLOCK + threadIdx.x;
-  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, false>(fin, ix, n, sn, tile + pf);
+  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, false, true>(fin, ix, n, sn, tile, pf);
   uint32_t off[Q];
   const bool live = x < n;
   // sites with an iolet link are stepped by the iolet warps
@@ -605,7 +609,7 @@ __global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_step2(const S* __res
   if (tile0 == kNoTile) return;
   const uint32_t tile = tile0 + j;
   const uint32_t x = pair_site(tile), y = x + 32;
-  if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, false>(fin, ix, n, sn, tile + pf);
+  if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, false, TILE_PAIRS>(fin, ix, n, sn, tile, pf);
   int32_t bs[CT_GROUPS];
   if (load_row_bases(ix, tile, bs)) {
     const uint32_t y1 = y < n ? y : x;  // a thread without a second site repeats its first, and does not store it
@@ -795,7 +799,7 @@ __global__ void __launch_bounds__(BLOCK, WIDE ? 4 : 5) k_aa_odd(S* A, const Inde
   using R = typename Real<S>::type;
   const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
   const uint32_t x = blockIdx.x * BLOCK + threadIdx.x;
-  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, true>(A, ix, n, sn, blockIdx.x + pf);
+  if (CT && pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) >= 4, true, true>(A, ix, n, sn, blockIdx.x, pf);
   int32_t code[Q];
   if (x < n) load_codes<CT, WIDE, LD_NC>(ix, sn, x, blockIdx.x, code);
   pdl_wait();
@@ -830,7 +834,7 @@ __global__ void __launch_bounds__(PAIR, pair_blocks<S>()) k_aa_odd2(S* A, const 
   if (aa_iolet_block<S, true, GRID>(A, io, p, &tile)) return;
   const uint32_t n = (uint32_t)p.n, sn = (uint32_t)p.sn;
   const uint32_t x = pair_site(tile), y = x + 32;
-  if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, true>(A, ix, n, sn, tile + pf);
+  if (pf && threadIdx.x < 32) prefetch_tile<S, sizeof(S) == 4, true, false>(A, ix, n, sn, tile, pf);
   int32_t bs[CT_GROUPS];
   if (load_row_bases(ix, tile, bs)) {
     const uint32_t y1 = y < n ? y : x;  // a thread without a second site repeats its first, and does not store it
@@ -1284,6 +1288,7 @@ inline unsigned iolet_blocks(const hlb_solver* h, int threads) {
 // Prefetch distance of the two-site kernels, in tiles.  An FP32 state that stays
 // in L2 has nothing to fetch ahead, and the hints for its rows only cost: none
 // below 600k sites.
+inline uint32_t prefetch_form(const hlb_solver* h) { return h->offset_major ? kPrefetchOffsets : 0u; }
 template <typename S>
 uint32_t pair_prefetch(const hlb_solver* h) {
   return sizeof(S) == 4 && h->n < 600000 ? 0u : (uint32_t)h->n_sm * 3u;
@@ -1357,7 +1362,8 @@ cudaError_t launch_gather(const hlb_solver* h, const void* fin, void* fout, cons
       auto kernel = pair_tiles<S>(h) ? (h->off32 ? k_step2<S, false, true> : k_step2<S, true, true>)
                                      : (h->off32 ? k_step2<S, false, false> : k_step2<S, true, false>);
       return launch_pdl(kernel, grid, PAIR, s, (const S*)fin, (S*)fout, h->index(),
-                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, spread, pair_prefetch<S>(h), tile0, p);
+                        h->d_links, h->d_amp, h->d_iolet_sites, h->n_iolet_sites, spread,
+                        pair_prefetch<S>(h) ? pair_prefetch<S>(h) | prefetch_form(h) : 0u, tile0, p);
     }
   }
   const unsigned grid = whole ? spread_iolets(h, BLOCK, BLOCK, &spread)
@@ -1367,7 +1373,7 @@ cudaError_t launch_gather(const hlb_solver* h, const void* fin, void* fout, cons
   auto kernel = h->compact ? (h->off32 ? k_step<S, false, CT> : k_step<S, true, CT>)
                            : (h->off32 ? k_step<S, false, false> : k_step<S, true, false>);
   return launch_pdl(kernel, grid, BLOCK, s, (const S*)fin, (S*)fout, h->index(), h->d_links, h->d_amp,
-                    h->d_iolet_sites, h->n_iolet_sites, spread, (uint32_t)h->n_sm * 5u, tile0, p);
+                    h->d_iolet_sites, h->n_iolet_sites, spread, (uint32_t)h->n_sm * 5u | prefetch_form(h), tile0, p);
 }
 
 template <typename S>
@@ -1417,13 +1423,13 @@ cudaError_t launch_aa(const hlb_solver* h, S* A, bool odd, const StepParams& p, 
                                         : !h->offset_major && h->n >= kOddPairSites)) {
         const AAIolets io = aa_iolets<GRID>(h, g, PAIR);
         return launch_pdl(h->off32 ? k_aa_odd2<S, false, GRID> : k_aa_odd2<S, true, GRID>, g + io.blocks, PAIR, s, A,
-                          h->index(), io, pair_prefetch<S>(h), p);
+                          h->index(), io, h->offset_major ? 0u : pair_prefetch<S>(h), p);
       }
     }
     if constexpr (!GRID) {
       return launch_pdl(h->compact ? (h->off32 ? k_aa_odd<S, false, true> : k_aa_odd<S, true, true>)
                                    : (h->off32 ? k_aa_odd<S, false, false> : k_aa_odd<S, true, false>),
-                        g, BLOCK, s, A, h->index(), (uint32_t)h->n_sm * (h->off32 ? 3u : 4u), p);
+                        g, BLOCK, s, A, h->index(), (uint32_t)h->n_sm * (h->off32 ? 3u : 4u) | prefetch_form(h), p);
     }
     return cudaErrorInvalidValue;  // GRID: compact FP32
   }

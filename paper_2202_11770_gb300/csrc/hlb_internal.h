@@ -113,7 +113,7 @@ struct hlb_solver {
   int64_t n_ilist = 0;                // entries of d_ilist
   int64_t red_slots = 0;
 
-  hlb::IndexTables index() const { return {d_src, d_ctab, d_tbase, d_rtab, d_rbase, d_imask, offset_major ? 1 : 0}; }
+  hlb::IndexTables index() const { return {d_src, d_ctab, d_tbase, d_rtab, d_rbase, d_imask}; }
   size_t elem_bytes() const;
   size_t state_bytes() const { return elem_bytes() * 19 * (size_t)n; }
   // kernel parameters for a launch that gathers with boundary data at time tb
