@@ -84,7 +84,7 @@ CTYPE = {"fp32": "float", "bf16": "__nv_bfloat16", "fp16": "__half", "fp64": "do
 # DRAM traffic per site update from one ncu capture (profiles/), valid only
 # while the kernel sources hash to the recorded value.
 TRAFFIC_FILES = ["paper_2202_11770_gb300/csrc/hlb_common.cuh", "paper_2202_11770_gb300/csrc/hlb_forward.cu"]
-TRAFFIC = {"sha": "477006fe2bec94ea",
+TRAFFIC = {"sha": "e4831f67c3d588a7",
            # ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch (mean of two), 20,000,864-site
            # tree, FP32, kernels on the row form of the compact index table with the L2 prefetch
            "index": "compact",

@@ -820,8 +820,8 @@ __device__ __forceinline__ double wk_advance(double Rp, double C, double Rd, dou
   *rho_c += (q - (*rho_c - rho_d) / Rd) / C;
   return fmadd(Rp, q, *rho_c) - 1.0;
 }
-// An outlet's link masses are summed by this many lanes, lane l its links l,
-// l + kWkLanes, .. in order, then the lanes of a warp, then the warps.
+// In the pull scheme an outlet's link masses are summed by this many lanes, lane l
+// its links l, l + kWkLanes, .. in order, then the lanes of a warp, then the warps.
 constexpr int kWkLanes = 64;
 
 // Sites a thread of a mass reduction over a lattice of n takes (a block: that

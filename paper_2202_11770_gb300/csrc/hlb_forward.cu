@@ -68,8 +68,9 @@ __device__ __forceinline__ void l2_prefetch(const void* q, uint32_t bytes) {
 // lattice is left to its own loads: where most tiles have the offset form, the
 // index words are its nine rows (lanes 0-8) and the bases its own (kPrefetchOffsets
 // in `pf`; OFFSETS: asked at all, which the small-lattice form of k_step2 is not:
-// the longer code made some of its steps 3 to 10 % slower).  Every range is clamped to its array: rtab holds CT_ROW_WORDS rows of sn words, ctab nine,
-// A 19 rows of n populations.
+// the longer code made some of its steps 3 to 10 % slower).  Every range is
+// clamped to its array: rtab holds CT_ROW_WORDS rows of sn words, ctab nine, A 19
+// rows of n populations.
 constexpr uint32_t kPrefetchOffsets = 0x80000000u;
 template <typename S, bool POPS, bool ROWOPP, bool OFFSETS>
 __device__ __forceinline__ void prefetch_tile(const S* A, const IndexTables& ix, uint32_t n, uint32_t sn,
@@ -90,7 +91,7 @@ __device__ __forceinline__ void prefetch_tile(const S* A, const IndexTables& ix,
     // row_group(i) of a run-time direction
     const int g = z == 0 ? (y > 0 ? 0 : 1) : (y == 0 ? (z > 0 ? 2 : 3) : (z > 0 ? (y > 0 ? 4 : 7) : (y > 0 ? 6 : 5)));
     const int64_t first = offsets ? __ldg(ix.tbase + (uint64_t)tile * CT_BASES + (i - 1))
-                                          : (int64_t)x0 - k_cx[i] + ((y | z) ? __ldg(rb + g) : 0);
+                                  : (int64_t)x0 - k_cx[i] + ((y | z) ? __ldg(rb + g) : 0);
     const uint64_t b = first > 0 ? (uint64_t)first : 0;
     const uint64_t r = ROWOPP ? (uint64_t)lane_opp(i) : (uint64_t)i;
     const uint64_t e = b + 320 < (uint64_t)n ? b + 320 : (uint64_t)n;
@@ -1495,10 +1496,10 @@ __global__ void __launch_bounds__(BLOCK) k_wk_update(const S* __restrict__ fin, 
                                                      const double* __restrict__ par, double* __restrict__ state,
                                                      double* ioval, double* __restrict__ iovnext, int shift) {
   using R = typename Real<S>::type;
-  // Links between two block barriers.  FP32 AA steps of 50k sites with outlets 7.9
-  // us at two a thread, 8.3 at one; at four (8 KB) the FP64 pull step, which lasts
-  // as long as the SM that gets most blocks, took 50 to 70 us instead of 42.
-  constexpr int CHUNK = 2 * BLOCK;
+  // Links between two block barriers (pull).  50k sites with outlets, single steps:
+  // FP32 10.8 us at one a thread, 10.6 at two and four; FP64 42 us at one and two, 50
+  // to 70 at four (8 KB: it lasts as long as the SM that gets most blocks).
+  constexpr int CHUNK = AA ? 1 : 2 * BLOCK;
   __shared__ double sh[BLOCK / 32], mass[CHUNK];
   const int k = blockIdx.x;
   pdl_wait();
@@ -1510,14 +1511,12 @@ __global__ void __launch_bounds__(BLOCK) k_wk_update(const S* __restrict__ fin, 
   }
   const int64_t n = p.n;
   double acc = 0;
-  for (int64_t r0 = begin[k], end = begin[k + 1]; r0 < end; r0 += CHUNK) {
+  if (AA)  // no multi-step launches, so no order to keep to: all threads add
+    for (int64_t r = begin[k] + threadIdx.x; r < begin[k + 1]; r += BLOCK) acc += lflux[r];
+  for (int64_t r0 = begin[k], end = AA ? r0 : begin[k + 1]; r0 < end; r0 += CHUNK) {
     const int count = (int)min((int64_t)CHUNK, end - r0);
     for (int m = threadIdx.x; m < count; m += BLOCK) {
       const int64_t r = r0 + m;
-      if (AA) {
-        mass[m] = lflux[r];
-        continue;
-      }
       const LinkRec L = links[r];
       const int64_t x = L.site;
       R own[Q];
@@ -1615,6 +1614,7 @@ struct ReduceOp {
                                       : launch_sums<S, M, false>(h, (const S*)fin, p, totals, links, monitor, s)));
     const int K = h->n_iolets;
     const int64_t* begin = (const int64_t*)(h->d_red + hlb_reduce_partials(h->n));  // link ranges stored after the partials
+    if (const cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
     // programmatic launch: its blocks are there when k_sums ends (monitor of 45k sites without fluxes 29 -> 27 us)
     return launch_pdl(
         k_sums_finish, (unsigned)(monitor ? 1 + 2 * K : 1 + K), 512, s, h->d_red, totals ? mass_blocks(owned, mass_sites(h->n)) : 0, owned, K, h->d_lflux, begin, totals && have_flux ? 1 : 0, h->d_msite, h->d_ioff, out, out + 1 + K);
